@@ -280,10 +280,10 @@ void heat_destroy_server(heat_server* srv);
  * that status and the requests already running continue undisturbed. n = 0
  * clears the hook. */
 heat_status heat_debug_fail_engine_builds(int n);
-/* Testing hook for the bounded waits of the persistent iteration (tuning
- * loop): engines built or refreshed afterwards expect extra_arrivals (0 or 1)
- * arrivals at each grid barrier beyond their grid, so with 1 no barrier ever
- * completes, and bound one wait by limit_s seconds (0: the engine's own
+/* Testing hook for the bounded waits of the persistent kernels (tuning loop,
+ * and the on-chip solve of variants 0 and -1): engines built or refreshed
+ * afterwards expect extra_arrivals (0 or 1) arrivals at each grid barrier or
+ * all-sum beyond their blocks, so with 1 no wait ever completes, and bound one wait by limit_s seconds (0: the engine's own
  * bound of 1 s plus 50 ns per node). A wait that runs out ends the kernel;
  * the step then fails with HEAT_ERR_TIMEOUT and the GPU context stays
  * usable. HEAT_ERR_ARG unless extra_arrivals is 0 or 1 and
@@ -536,7 +536,13 @@ heat_status heat_probe_grid_barrier(int blocks_per_sm, int reps, double* us_per_
  * any batch built under the same table.
  *   variant[p]: for heat_precision p, the warp-segment apply kernel variant
  *     (0 .. heat_tuning_num_variants()-1) or -1 for the block-tile apply.
- *     Default {-1, 0, 0}.
+ *     Default {-1, 0, 0}. Under variant 0 (FP32 paths) and -1 (FP64) a mesh
+ *     that fits the GPU's shared memory (about 1.1 million nodes in FP32,
+ *     130,000 in FP64) runs its whole inner solve in one persistent
+ *     cooperative launch instead; larger meshes and Chebyshev members take
+ *     the streaming kernels. Its waits are bounded like the grid barrier's
+ *     (see loop): one that runs out fails the simulation with
+ *     HEAT_ERR_TIMEOUT.
  *   seg_nodes[b]: output nodes per warp-segment tile for meshes of bucket b
  *     (N < 200000, N < 4000000, larger); 32 .. 2^20, default 512.
  *   pw_quads[p]: for heat_precision p, groups of 4 nodes each thread of the

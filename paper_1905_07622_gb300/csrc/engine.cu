@@ -11,12 +11,15 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <mutex>
+#include <tuple>
 #include <type_traits>
 
 #include "engine.h"
 #include "loop_kernels.cuh"
 #include "open_kernels.cuh"
+#include "res_kernels.cuh"
 
 namespace heat {
 
@@ -44,6 +47,10 @@ struct KernelSet {
   // the CG iterations of a tick as one persistent kernel (replaces the
   // apply and update launches when set; FP32 paths, register-prefetch apply)
   LoopFn loop = nullptr;
+  // the inner solve held on the chip: iterates the members whose mesh fits
+  // (SimDev::res.g > 0); the others take apply and update
+  ResFn res = nullptr;
+  int res_blocks = 0, res_smem = 0;  // resident blocks, dynamic shared memory limit
 };
 
 // The warp-segment forms of k_open (tuning open_w): 32-lane segments of 2
@@ -87,6 +94,7 @@ struct WVariant {
   int smem32, smem64;  // dynamic shared memory per block
   bool fused;          // FP32 only: the fused iteration kernel k_cg_iter
   TileFn cheb32[2], cheb64[2];  // Chebyshev passes of this segment shape (null: fused)
+  bool res = false;    // FP32 only: meshes that fit iterate on the chip (k_cg_res)
 };
 // One register-prefetch Chebyshev pass kernel per segment shape and type,
 // bounded like that shape's register-prefetch apply (FP64: one block per SM).
@@ -126,13 +134,20 @@ static constexpr WVariant wv_fused() {
   return {SX, NY, W, 0, {k_cg_iter<SX, NY, W, MINB, E_Q1>, k_cg_iter<SX, NY, W, MINB, E_P1>}, {nullptr, nullptr},
           0,  0,  true, {nullptr, nullptr}, {nullptr, nullptr}};
 }
+// the on-chip inner solve where the mesh fits, this streaming shape elsewhere
+template <int SX, int NY, int W, int MINB>
+static constexpr WVariant wv_res() {
+  WVariant v = wv<SX, NY, W, 0, MINB, 0>();
+  v.res = true;
+  return v;
+}
 // (segment width, rows, warps, stages, min blocks per SM for float / double,
 // 0 = no double kernel)
 static const WVariant kVariants[] = {
-    wv<16, 4, 4, 0, 3, 0>(), wv<32, 4, 4, 0, 3, 0>(), wv<16, 2, 8, 0, 2, 1>(), wv<32, 2, 4, 0, 4, 1>(),
+    wv_res<16, 4, 4, 3>(), wv<32, 4, 4, 0, 3, 0>(), wv<16, 2, 8, 0, 2, 1>(), wv<32, 2, 4, 0, 4, 1>(),
     wv<16, 4, 4, 3, 4, 0>(), wv<32, 4, 4, 3, 4, 0>(), wv<16, 2, 8, 3, 2, 1>(), wv<32, 4, 4, 3, 3, 0>(),
     wv<32, 4, 4, 4, 3, 0>(),     wv_fused<16, 4, 4, 2>(), wv_fused<32, 4, 4, 2>(), wv_fused<16, 4, 4, 3>(),
-    wv_fused<32, 4, 4, 3>(),     wv_fused<16, 2, 8, 2>(), wv_fused<32, 2, 4, 4>(),
+    wv_fused<32, 4, 4, 3>(),     wv_fused<16, 2, 8, 2>(), wv_fused<32, 2, 4, 4>(), wv<16, 4, 4, 0, 3, 0>(),
 };
 constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
 
@@ -152,7 +167,7 @@ bool variant_info(int v, int info[6]) {
   info[2] = kVariants[v].warps;
   info[3] = kVariants[v].f64[0] != nullptr;
   info[4] = kVariants[v].stages;
-  info[5] = kVariants[v].fused;
+  info[5] = kVariants[v].fused || kVariants[v].res;  // one kernel runs whole iterations
   return true;
 }
 
@@ -200,6 +215,138 @@ static TileFn update_kernel(int prec, int qpt) {
 
 static int sm_count();
 
+// ------------------------------------------------- the on-chip inner solve
+
+// k_cg_res of this precision and element, when the device can run it: one
+// block per SM, all resident at once (a cooperative launch).
+static void res_kernel_set(KernelSet& k, bool fp64, int elem) {
+  int dev = 0, coop = 0, optin = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  k.res = nullptr;
+  if (!coop || optin < 96 * 1024) {
+    cudaGetLastError();
+    return;
+  }
+  ResFn fn = res_kernel(fp64, elem);
+  cudaFuncAttributes fa;
+  if (cudaFuncGetAttributes(&fa, (const void*)fn) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  const int smem = (optin - (int)fa.sharedSizeBytes) & ~15;
+  if (cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  k.res = fn;
+  k.res_smem = smem;
+  k.res_blocks = sm_count();
+}
+
+static int res_nodes(const ResGeo& r) { return r.bx * r.by * r.bz; }
+
+// Estimated cycles of one iteration on boxes r, fitted to clock readings in
+// the kernel (boxes of 16^3 to 105^3 meshes): a march layer takes a warp 850
+// cycles alone on its scheduler and 690 beside others, a pointwise group of
+// 4 nodes per thread 640 over the passes, an all-sum about 3,000 with its
+// block barriers.
+static double res_cycles(const ResGeo& r, bool fp64) {
+  const double sums = r.g > 1 ? 6200.0 + 5.0 * r.g : 2600.0;
+  if (fp64) {
+    // a warp's FP64 instruction takes its scheduler 64 cycles; 27 + 6 of them per node and iteration
+    const int warps = (res_nodes(r) + 31) / 32;
+    return ((warps + 3) / 4) * 33.0 * 64.0 + 3000.0 + sums;
+  }
+  const ResLayout l = res_layout(r, false);
+  const int pairs = (l.nseg * l.nyt + 1) / 2, chunks = (r.bz + r.zc - 1) / r.zc;
+  const int per_sched = (pairs * chunks + 3) / 4;
+  const double march = (r.zc + 1.3) * (per_sched > 1 ? 690.0 * per_sched : 850.0);
+  return march + res_groups(r) * 640.0 + 900.0 + sums;
+}
+
+// The boxes of one simulation (res.g = 0: it does not fit or gains nothing).
+// FP32: the least time^2 x blocks, halfway between the fastest simulation
+// alone (all SMs) and the most simulations side by side (fewest SMs each).
+// FP64 runs at 1/58 of the FP32 rate, so its time is arithmetic spread over
+// the SMs: the fastest alone is also the best in a batch. A function of the
+// mesh and the GPU only, so results are the same alone and in a batch.
+static ResGeo res_search(int X, int Y, int Z, int max_blocks, int smem, bool fp64) {
+  ResGeo best{};
+  double best_cost = 1e300;
+  auto ceil_div = [](int a, int b) { return (a + b - 1) / b; };
+  for (int gz = 1, last_z = 0; gz <= std::min(Z, max_blocks); ++gz) {
+    const int bz = ceil_div(Z, gz);
+    if (bz == last_z) continue;
+    last_z = bz;
+    for (int gy = 1, last_y = 0; gy <= Y && ceil_div(Z, bz) * gy <= max_blocks; ++gy) {
+      const int by = ceil_div(Y, gy);
+      if (by == last_y) continue;
+      last_y = by;
+      for (int gx = 1, last_x = 0; gx <= 8; ++gx) {
+        int bx = ceil_div(X, gx);
+        if (gx > 1) bx = (bx + 3) & ~3;  // exchanged groups of 4 start at multiples of 4
+        if (bx == last_x) continue;
+        last_x = bx;
+        ResGeo r{};
+        r.gx = ceil_div(X, bx);
+        r.gy = ceil_div(Y, by);
+        r.gz = ceil_div(Z, bz);
+        r.g = r.gx * r.gy * r.gz;
+        r.bx = bx;
+        r.by = by;
+        r.bz = bz;
+        r.zc = bz;
+        if (r.g > max_blocks) continue;
+        if (fp64 ? res_nodes(r) > kResMaxN * kResThreads : res_groups(r) > kResMaxQ) continue;
+        if (res_layout(r, fp64).bytes > smem) continue;
+        for (int chunks = 1; chunks <= (fp64 ? 1 : std::min(8, bz)); ++chunks) {
+          r.zc = ceil_div(bz, chunks);
+          const double t = res_cycles(r, fp64), cost = fp64 ? t : t * t * r.g;
+          if (cost < best_cost) {
+            best_cost = cost;
+            best = r;
+          }
+        }
+      }
+    }
+  }
+  return best;
+}
+
+static ResGeo res_plan(const SimDev& d, const KernelSet& ks, bool fp64) {
+  if (!ks.res || d.cheb_m >= 2) return ResGeo{};  // Chebyshev passes run on the streaming kernels
+  using Key = std::tuple<int, int, int, int, int, bool>;
+  static std::mutex mu;
+  static std::map<Key, ResGeo> plans;  // searched once per mesh size, bounded
+  const Key key{d.nx, d.ny, d.nz, ks.res_blocks, ks.res_smem, fp64};
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = plans.find(key);
+  if (it != plans.end()) return it->second;
+  const ResGeo r = res_search(d.nx + 1, d.ny + 1, d.nz + 1, ks.res_blocks, ks.res_smem, fp64);
+  if (plans.size() >= 1024) plans.clear();
+  plans[key] = r;
+  return r;
+}
+
+// Bytes of a simulation's exchange area and where its parts start.
+struct ResBytes {
+  size_t z, x, slots, tag, total;
+};
+static ResBytes res_bytes(const SimDev& d, bool fp64) {
+  ResBytes b{};
+  if (d.res.g < 1) return b;
+  auto up = [](size_t n) { return (n + 255) & ~(size_t)255; };
+  b.z = 0;
+  const size_t nz = d.res.g > 1 ? (size_t)((d.nx + 4) & ~3) * (d.ny + 1) * (d.nz + 1) * (fp64 ? 16 : 8) : 0;
+  b.x = up(nz);
+  b.slots = b.x + (fp64 ? 0 : (size_t)d.res.g * 2 * res_groups(d.res) * kResThreads * sizeof(float4));
+  b.tag = b.slots + up(2 * (size_t)res_mail(d.res.g) * sizeof(ulonglong2));
+  b.total = b.tag + 256;
+  return b;
+}
+
 // The kernels of precision prec under tuning table t. With Chebyshev passes
 // (cheb) a fused variant is replaced by the register-prefetch variant of the
 // same segment shape: the fused iteration has no place for the passes.
@@ -238,10 +385,12 @@ static KernelSet kernel_set(int prec, const Tuning& t, bool cheb = false, int el
         cudaFuncSetAttribute(k.apply_w, cudaFuncAttributeMaxDynamicSharedMemorySize, k.apply_w_smem);
       // the persistent iteration: FP32 paths, trilinear boxes, register
       // prefetch, separate update, no Chebyshev passes
-      if (t.loop[prec] && prec != P_FP64 && elem == E_Q1 && !cheb && !v.fused && v.stages == 0)
+      if (t.loop[prec] && prec != P_FP64 && elem == E_Q1 && !cheb && !v.fused && !v.res && v.stages == 0)
         k.loop = loop_kernel(v.sx, v.ny, v.warps, t.pw_quads[prec]);
+      if (v.res) res_kernel_set(k, false, elem);
     }
   }
+  if (prec == P_FP64 && variant < 0) res_kernel_set(k, true, elem);
   if (elem == E_Q1 && t.open_w[prec]) {
     k.open_w = open_w_kernel(prec, t.open_w[prec]);
     k.owsx = kOpenSX;
@@ -317,6 +466,16 @@ struct Engine {
   int phases_cap = 0;
   std::vector<SimDev> h_sims;
   std::vector<int2> h_op, h_pw;
+  // on-chip solve (ks.res): exchange areas, each block's tasks
+  unsigned char* d_res = nullptr;
+  int* d_res_off = nullptr;
+  int2* d_res_tasks = nullptr;
+  size_t cap_res = 0;
+  long long cap_tasks = 0;
+  int grid_res = 0, smem_res = 0;
+  bool has_res = false, has_stream = true;  // members on the chip / on the streaming kernels
+  std::vector<int> h_res_off;
+  std::vector<int2> h_res_tasks;
   long long cap_sims = 0;   // simulations the descriptor array holds
   bool grid_cap = false;    // grids sized by the capacities (members can change without a new graph)
 };
@@ -335,12 +494,13 @@ static bool injected_failure() {
 // apply + update, or the fused kernel; or k_open and the persistent loop.
 static int tick_launches(const Engine* e) {
   if (e->ks.loop) return 2;
-  return 1 + (e->ncheb + (e->ks.fused ? 1 : 2)) * e->iters_per_tick;
+  return 1 + (e->has_res ? 1 : 0) + (e->has_stream ? (e->ncheb + (e->ks.fused ? 1 : 2)) * e->iters_per_tick : 0);
 }
 
 // Rounds (CG iterations) one persistent launch runs at most: a solve's
 // inner iterations normally end it first, at a phase change.
 constexpr int kLoopRounds = 256;
+constexpr int kResRounds = 4096;
 
 // Test hook (heat_debug_loop_wait): arrivals the barrier expects beyond the
 // grid, and the bound of one wait in ns (0: the engine's own bound).
@@ -350,8 +510,9 @@ static std::atomic<unsigned long long> g_loop_limit_ns{0};
 // Barrier state for a fresh launch. One wait is bounded by 1 s plus 50 ns
 // per node of the members (a phase of the largest batches takes far less),
 // or by the test hook's bound; a launch runs at most `rounds` iterations.
-static heat_status loop_sync_reset(Engine* e, int rounds = kLoopRounds) {
+static heat_status loop_sync_reset(Engine* e, int rounds = 0) {
   if (!e->d_sync) return HEAT_OK;
+  if (rounds == 0) rounds = e->ks.loop ? kLoopRounds : kResRounds;
   long long nodes = 0;
   for (const heat_sim* s : e->sims) nodes += s->nn;
   GridSync g{};
@@ -381,6 +542,7 @@ static heat_status loop_abort(Engine* e) {
     if (st != HEAT_OK) return st;
   }
   e->h_abort[0] = e->h_abort[1] = 0;
+  if (e->d_res) CUDA_TRY(cudaMemsetAsync(e->d_res, 0, e->cap_res, e->stream));  // no tag of the broken launch stays
   return loop_sync_reset(e);
 }
 
@@ -399,7 +561,8 @@ static int members_ncheb(const Engine* e) { return members_ncheb_of(e->sims.data
 // and with them the order of every reduction, are the same whether the
 // simulation runs alone or in a batch: its results are bitwise identical.
 constexpr long long kTileNodes = 2048;
-static void tile_geometry(SimDev& d, const KernelSet& ks) {
+static void tile_geometry(SimDev& d, const KernelSet& ks, bool fp64) {
+  d.res = res_plan(d, ks, fp64);
   d.ntx = (d.nx + 1 + ks.sx - 2) / (ks.sx - 1);
   d.nty = (d.ny + 1 + ks.sy - 2) / (ks.sy - 1);
   const int levels = d.nz + 1;
@@ -466,6 +629,53 @@ static int sm_count() {
   return sms;
 }
 
+// Deals the members on the chip to the blocks of k_cg_res. Every block runs
+// its tasks in member order, so the first unfinished member's blocks are all
+// at it and the launch always advances. Each member takes the blocks that
+// are free first.
+static heat_status res_schedule(Engine* e, bool has_res, bool has_stream, size_t res_used) {
+  e->has_res = has_res;
+  e->has_stream = has_stream;
+  e->grid_res = e->smem_res = 0;
+  if (!has_res) return HEAT_OK;
+  const int nb = e->ks.res_blocks;
+  const bool f64 = e->prec == P_FP64;
+  std::vector<std::vector<int2>> list(nb);
+  std::vector<double> load(nb, 0.0);
+  std::vector<int> order(nb);
+  int used = 0;
+  long long ntasks = 0;
+  for (size_t i = 0; i < e->h_sims.size(); ++i) {
+    const ResGeo& r = e->h_sims[i].res;
+    if (r.g == 0) continue;
+    for (int b = 0; b < nb; ++b) order[b] = b;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return load[a] < load[b]; });
+    const double end = load[order[r.g - 1]] + res_cycles(r, f64);
+    for (int k = 0; k < r.g; ++k) {
+      list[order[k]].push_back(make_int2((int)i, k));
+      load[order[k]] = end;
+      used = std::max(used, order[k] + 1);
+    }
+    ntasks += r.g;
+    e->smem_res = std::max(e->smem_res, res_layout(r, f64).bytes);
+  }
+  if (ntasks > e->cap_tasks) return set_error(HEAT_ERR_ARG, "engine: on-chip tasks exceed their capacity");
+  e->grid_res = e->grid_cap ? nb : used;
+  if (e->grid_cap) e->smem_res = e->ks.res_smem;
+  e->h_res_off.assign(1, 0);
+  e->h_res_tasks.clear();
+  for (int b = 0; b < nb; ++b) {
+    e->h_res_tasks.insert(e->h_res_tasks.end(), list[b].begin(), list[b].end());
+    e->h_res_off.push_back((int)e->h_res_tasks.size());
+  }
+  CUDA_TRY(cudaMemcpyAsync(e->d_res_off, e->h_res_off.data(), sizeof(int) * e->h_res_off.size(), cudaMemcpyHostToDevice,
+                           e->stream));
+  CUDA_TRY(cudaMemcpyAsync(e->d_res_tasks, e->h_res_tasks.data(), sizeof(int2) * e->h_res_tasks.size(),
+                           cudaMemcpyHostToDevice, e->stream));
+  CUDA_TRY(cudaMemsetAsync(e->d_res, 0, res_used, e->stream));  // tags start anew with the areas
+  return HEAT_OK;
+}
+
 static heat_status engine_upload(Engine* e) {
   e->h_sims.clear();
   e->h_op.clear();
@@ -474,18 +684,39 @@ static heat_status engine_upload(Engine* e) {
   e->h_ow.clear();
   const int sms = sm_count();
   long long item_base = 0;
+  size_t res_base = 0;
+  const bool f64 = e->prec == P_FP64;
+  bool has_res = false, has_stream = false;
   for (size_t i = 0; i < e->sims.size(); ++i) {
     SimDev d = e->sims[i]->dev;
-    tile_geometry(d, e->ks);
+    tile_geometry(d, e->ks, e->prec == P_FP64);
     d.fused = e->ks.fused ? 1 : 0;
     d.partial = e->d_partial + 4 * item_base;
     item_base += std::max(std::max(std::max(d.ntiles, d.npw), d.w_items), d.o_items);
-    for (int t = 0; t < d.ntiles; ++t) e->h_op.push_back(make_int2((int)i, t));
-    for (int t = 0; t < d.npw; ++t) e->h_pw.push_back(make_int2((int)i, t));
-    for (int t = 0; t < d.w_items; ++t) e->h_aw.push_back(make_int2((int)i, t));
+    const bool stream = d.res.g == 0;
+    // the block tiles also carry k_open's passes (k_apply_dot skips members on the chip)
+    if (stream || !e->ks.open_w)
+      for (int t = 0; t < d.ntiles; ++t) e->h_op.push_back(make_int2((int)i, t));
+    if (stream) {
+      for (int t = 0; t < d.npw; ++t) e->h_pw.push_back(make_int2((int)i, t));
+      for (int t = 0; t < d.w_items; ++t) e->h_aw.push_back(make_int2((int)i, t));
+    }
     for (int t = 0; t < d.o_items; ++t) e->h_ow.push_back(make_int2((int)i, t));
+    (stream ? has_stream : has_res) = true;
+    if (!stream) {
+      const ResBytes rb = res_bytes(d, f64);
+      if (res_base + rb.total > e->cap_res) return set_error(HEAT_ERR_ARG, "engine: exchange areas exceed their capacity");
+      unsigned char* p = e->d_res + res_base;
+      d.res_z = p + rb.z;
+      d.res_x = p + rb.x;
+      d.res_slots = (ulonglong2*)(p + rb.slots);
+      d.res_tag = (unsigned int*)(p + rb.tag);
+      res_base += rb.total;
+    }
     e->h_sims.push_back(d);
   }
+  heat_status rst = res_schedule(e, has_res, has_stream, res_base);
+  if (rst != HEAT_OK) return rst;
   if ((long long)e->h_op.size() > e->cap_op || (long long)e->h_pw.size() > e->cap_pw ||
       (long long)e->h_aw.size() > e->cap_aw || (long long)e->h_ow.size() > e->cap_ow ||
       item_base > e->cap_partial)
@@ -493,10 +724,12 @@ static heat_status engine_upload(Engine* e) {
   const int nwork[4] = {(int)e->h_op.size(), (int)e->h_pw.size(), (int)e->h_aw.size(), (int)e->h_ow.size()};
   CUDA_TRY(cudaMemcpyAsync(e->d_sims, e->h_sims.data(), sizeof(SimDev) * e->h_sims.size(), cudaMemcpyHostToDevice,
                            e->stream));
-  CUDA_TRY(cudaMemcpyAsync(e->d_work_op, e->h_op.data(), sizeof(int2) * e->h_op.size(), cudaMemcpyHostToDevice,
-                           e->stream));
-  CUDA_TRY(cudaMemcpyAsync(e->d_work_pw, e->h_pw.data(), sizeof(int2) * e->h_pw.size(), cudaMemcpyHostToDevice,
-                           e->stream));
+  if (!e->h_op.empty())
+    CUDA_TRY(cudaMemcpyAsync(e->d_work_op, e->h_op.data(), sizeof(int2) * e->h_op.size(), cudaMemcpyHostToDevice,
+                             e->stream));
+  if (!e->h_pw.empty())
+    CUDA_TRY(cudaMemcpyAsync(e->d_work_pw, e->h_pw.data(), sizeof(int2) * e->h_pw.size(), cudaMemcpyHostToDevice,
+                             e->stream));
   if (!e->h_aw.empty())
     CUDA_TRY(cudaMemcpyAsync(e->d_work_aw, e->h_aw.data(), sizeof(int2) * e->h_aw.size(), cudaMemcpyHostToDevice,
                              e->stream));
@@ -558,6 +791,22 @@ static void apply_launch(const Engine* e, TileFn* fn, int* grid, int* threads, c
   }
 }
 
+// One launch of the on-chip solve: cooperative, all blocks resident.
+static cudaError_t res_launch(Engine* e, cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(e->grid_res);
+  cfg.blockDim = dim3(kResThreads);
+  cfg.dynamicSmemBytes = (size_t)e->smem_res;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, e->ks.res, (const SimDev*)e->d_sims, (const int*)e->d_res_off,
+                            (const int2*)e->d_res_tasks, e->d_sync);
+}
+
 static heat_status engine_capture(Engine* e) {
   if (e->gexec) {
     cudaGraphExecDestroy(e->gexec);
@@ -613,7 +862,8 @@ static heat_status engine_capture(Engine* e) {
       lerr = cudaLaunchKernelEx(&cfg, e->ks.loop, (const SimDev*)e->d_sims, (const int2*)e->d_work_aw,
                                 (const int2*)e->d_work_pw, (const int*)e->d_nwork, e->d_sync);
     }
-    for (int it = 0; it < (e->ks.loop ? 0 : e->iters_per_tick) && lerr == cudaSuccess; ++it) {
+    if (e->has_res && lerr == cudaSuccess) lerr = res_launch(e, cap);
+    for (int it = 0; it < (e->ks.loop || !e->has_stream ? 0 : e->iters_per_tick) && lerr == cudaSuccess; ++it) {
       for (int k = 0; k < e->ncheb && lerr == cudaSuccess; ++k) {
         if (e->ks.cheb_w) lerr = launch(e->ks.cheb_w, e->grid_ch, 32 * e->ks.wwarps, e->d_work_aw, e->d_nwork + 2, 0);
         else lerr = launch(e->ks.cheb, e->grid_ch, e->ks.apply_threads, e->d_work_op, e->d_nwork, 0);
@@ -654,15 +904,20 @@ heat_status engine_create(heat_sim* const* sims, int nsims, int precision, cudaS
   e->ks = kernel_set(precision, tun ? *tun : tuning_get(), e->ncheb > 0, e->elem);
   e->stream = stream;
   // capacities: the geometry is a function of each mesh, so compute it
-  long long cap_op = 0, cap_pw = 0, cap_aw = 0, cap_ow = 0, cap_partial = 0;
+  long long cap_op = 0, cap_pw = 0, cap_aw = 0, cap_ow = 0, cap_partial = 0, cap_tasks = 0;
+  size_t cap_res = 0;
   for (heat_sim* s : e->sims) {
     SimDev d = s->dev;
-    tile_geometry(d, e->ks);
+    tile_geometry(d, e->ks, e->prec == P_FP64);
     cap_op += d.ntiles;
     cap_pw += d.npw;
     cap_aw += d.w_items;
     cap_ow += d.o_items;
     cap_partial += std::max(std::max(std::max(d.ntiles, d.npw), d.w_items), d.o_items);
+    d.cheb_m = 0;  // room for the on-chip solve also when the member starts with Chebyshev passes
+    d.res = res_plan(d, e->ks, precision == P_FP64);
+    cap_res += res_bytes(d, precision == P_FP64).total;
+    cap_tasks += d.res.g;
   }
   if (cap_op > (1LL << 30) || cap_pw > (1LL << 30) || cap_aw > (1LL << 30) || cap_ow > (1LL << 30)) {
     delete e;
@@ -681,6 +936,8 @@ heat_status engine_create(heat_sim* const* sims, int nsims, int precision, cudaS
   e->cap_aw = cap_aw;
   e->cap_ow = cap_ow;
   e->cap_partial = cap_partial;
+  e->cap_res = (size_t)grow((long long)cap_res);
+  e->cap_tasks = grow(cap_tasks);
   heat_status st = HEAT_OK;
   auto fail = [&](heat_status s) {
     engine_destroy(e);
@@ -697,6 +954,9 @@ heat_status engine_create(heat_sim* const* sims, int nsims, int precision, cudaS
       cudaMallocHost(&e->h_unfinished, 2 * sizeof(int)) != cudaSuccess ||
       cudaMalloc(&e->d_sync, sizeof(GridSync)) != cudaSuccess ||
       cudaMallocHost(&e->h_abort, 2 * sizeof(int)) != cudaSuccess ||
+      (e->cap_res > 0 && (cudaMalloc(&e->d_res, e->cap_res) != cudaSuccess ||
+                          cudaMalloc(&e->d_res_off, sizeof(int) * (e->ks.res_blocks + 1)) != cudaSuccess ||
+                          cudaMalloc(&e->d_res_tasks, sizeof(int2) * e->cap_tasks) != cudaSuccess)) ||
       cudaEventCreateWithFlags(&e->poll_ev[0], cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&e->poll_ev[1], cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
@@ -735,6 +995,9 @@ void engine_destroy(Engine* e) {
   cudaFree(e->d_unfinished);
   cudaFree(e->d_partial);
   if (e->d_sync) cudaFree(e->d_sync);
+  if (e->d_res) cudaFree(e->d_res);
+  if (e->d_res_off) cudaFree(e->d_res_off);
+  if (e->d_res_tasks) cudaFree(e->d_res_tasks);
   if (e->h_abort) cudaFreeHost(e->h_abort);
   if (e->h_unfinished) cudaFreeHost(e->h_unfinished);
   for (cudaEvent_t ev : e->poll_ev)
@@ -745,7 +1008,9 @@ void engine_destroy(Engine* e) {
 }
 
 heat_status engine_refresh(Engine* e) {
-  const int g_op = e->grid_op, g_pw = e->grid_pw, g_aw = e->grid_aw, g_ch = e->grid_ch;
+  const int g_op = e->grid_op, g_pw = e->grid_pw, g_aw = e->grid_aw, g_ch = e->grid_ch, g_ow = e->grid_ow;
+  const int g_res = e->grid_res, sm_res = e->smem_res;
+  const bool h_res = e->has_res, h_stream = e->has_stream;
   // a member's preconditioner may have changed: the passes per iteration, and
   // with them the kernel set (no fused iteration with passes) and the graph
   const int nch = members_ncheb(e);
@@ -766,7 +1031,9 @@ heat_status engine_refresh(Engine* e) {
   if (st != HEAT_OK) return st;
   st = loop_sync_reset(e);
   if (st != HEAT_OK) return st;
-  if (recapture || !e->gexec || e->grid_op != g_op || e->grid_pw != g_pw || e->grid_aw != g_aw || e->grid_ch != g_ch)
+  if (recapture || !e->gexec || e->grid_op != g_op || e->grid_pw != g_pw || e->grid_aw != g_aw || e->grid_ch != g_ch ||
+      e->grid_ow != g_ow || e->has_res != h_res || e->has_stream != h_stream || e->grid_res != g_res ||
+      e->smem_res != sm_res)
     return engine_capture(e);
   return HEAT_OK;
 }
@@ -774,20 +1041,24 @@ heat_status engine_refresh(Engine* e) {
 heat_status engine_set_members(Engine* e, heat_sim* const* sims, int nsims) {
   if (injected_failure()) return set_error(HEAT_ERR_NOMEM, "engine: update failure injected by the test hook");
   if (nsims < 1 || !sims || nsims > e->cap_sims) return set_error(HEAT_ERR_ARG, "engine: member set exceeds capacity");
-  long long op = 0, pw = 0, aw = 0, ow = 0, part = 0;
+  long long op = 0, pw = 0, aw = 0, ow = 0, part = 0, tasks = 0;
+  size_t res = 0;
   for (int i = 0; i < nsims; ++i) {
     const heat_sim* s = sims[i];
     if (s->prm.precision != e->prec || s->dev.elem != e->elem)
       return set_error(HEAT_ERR_ARG, "engine: a member's precision or element differs from the engine's");
     SimDev d = s->dev;
-    tile_geometry(d, e->ks);
+    tile_geometry(d, e->ks, e->prec == P_FP64);
     op += d.ntiles;
     pw += d.npw;
     aw += d.w_items;
     ow += d.o_items;
     part += std::max(std::max(std::max(d.ntiles, d.npw), d.w_items), d.o_items);
+    res += res_bytes(d, e->prec == P_FP64).total;
+    tasks += d.res.g;
   }
-  if (op > e->cap_op || pw > e->cap_pw || aw > e->cap_aw || ow > e->cap_ow || part > e->cap_partial)
+  if (op > e->cap_op || pw > e->cap_pw || aw > e->cap_aw || ow > e->cap_ow || part > e->cap_partial ||
+      res > e->cap_res || tasks > e->cap_tasks)
     return set_error(HEAT_ERR_ARG, "engine: member set exceeds the work-list capacity");
   // the last-block counters of newly added members start at zero
   for (int i = 0; i < nsims; ++i) {
@@ -805,7 +1076,8 @@ heat_status engine_set_members(Engine* e, heat_sim* const* sims, int nsims) {
 
 heat_status engine_step_all(Engine* e, int nsteps, heat_step_stats* stats, int reset_counters) {
   int max_iter = 1, max_outer = 1, poll = 32;
-  if (e->ks.loop) {  // the barrier bound and the test hook as they are now
+  const bool waits = e->ks.loop || e->has_res;  // kernels whose bounded waits can give up
+  if (waits) {  // the bound and the test hook as they are now
     heat_status st = loop_sync_reset(e);
     if (st != HEAT_OK) return st;
   }
@@ -831,7 +1103,8 @@ heat_status engine_step_all(Engine* e, int nsteps, heat_step_stats* stats, int r
     poll = std::min(poll, s->prm.poll_period);
   }
   // the persistent form polls after as many graph launches as the tick form
-  const int ticks_per_poll = std::max(1, poll / e->iters_per_tick);
+  // (on the chip a tick carries a whole inner solve: three ticks are a step)
+  const int ticks_per_poll = e->has_res && !e->has_stream ? 3 : std::max(1, poll / e->iters_per_tick);
   // Every tick advances each unfinished simulation by at least one CG
   // iteration or one phase change, so this bound is never reached by a
   // healthy solve; it turns a logic error into HEAT_ERR_TIMEOUT.
@@ -853,7 +1126,7 @@ heat_status engine_step_all(Engine* e, int nsteps, heat_step_stats* stats, int r
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaMemcpyAsync(e->h_unfinished + slot, e->d_unfinished + slot, sizeof(int), cudaMemcpyDeviceToHost,
                              e->stream));
-    if (e->ks.loop)
+    if (waits)
       CUDA_TRY(cudaMemcpyAsync(e->h_abort + slot, &e->d_sync->abort, sizeof(int), cudaMemcpyDeviceToHost, e->stream));
     CUDA_TRY(cudaEventRecord(e->poll_ev[slot], e->stream));
     long long waited = -1;  // the batch whose counts are read now
@@ -862,7 +1135,7 @@ heat_status engine_step_all(Engine* e, int nsteps, heat_step_stats* stats, int r
     if (waited < 0) continue;  // batch 1 queued right after batch 0 was read
     const int ws = (int)(waited & 1);
     CUDA_TRY(cudaEventSynchronize(e->poll_ev[ws]));
-    if (e->ks.loop && e->h_abort[ws]) {
+    if (waits && e->h_abort[ws]) {
       CUDA_TRY(cudaStreamSynchronize(e->stream));
       heat_status st = loop_abort(e);
       if (st != HEAT_OK) return st;
@@ -925,7 +1198,7 @@ heat_status engine_read_phases(Engine* e, int* phases) {
     e->phases_cap = n;
   }
   d = e->d_phases;
-  if (e->ks.loop) {  // a persistent launch that gave up fails the unfinished members first
+  if (e->ks.loop || e->has_res) {  // a persistent launch that gave up fails the unfinished members first
     CUDA_TRY(cudaMemcpyAsync(e->h_abort, &e->d_sync->abort, sizeof(int), cudaMemcpyDeviceToHost, e->stream));
     CUDA_TRY(cudaStreamSynchronize(e->stream));
     if (*e->h_abort) {
@@ -948,19 +1221,21 @@ size_t engine_footprint(long long nn, long long nx, long long ny, long long nz) 
   // the largest work lists any precision's kernels need under the current table
   const Tuning t = tuning_get();
   long long op = 0, pw = 0, aw = 0, ow = 0;
+  size_t res = 0;
   for (int p = 0; p < 3; ++p) {
     SimDev d{};
     d.nx = (int)nx;
     d.ny = (int)ny;
     d.nz = (int)nz;
     d.nn = nn;
-    tile_geometry(d, kernel_set(p, t));
+    tile_geometry(d, kernel_set(p, t), p == P_FP64);
+    res = std::max(res, res_bytes(d, p == P_FP64).total + sizeof(int2) * d.res.g);
     op = std::max<long long>(op, d.ntiles);
     pw = std::max<long long>(pw, d.npw);
     aw = std::max<long long>(aw, d.w_items);
     ow = std::max<long long>(ow, d.o_items);
   }
-  return (size_t)(sizeof(int2) * (op + pw + aw + ow) +
+  return res + (size_t)(sizeof(int2) * (op + pw + aw + ow) +
                   sizeof(double) * 4 * std::max(std::max(std::max(op, pw), aw), ow) + sizeof(SimDev) + 64);
 }
 
@@ -1039,7 +1314,7 @@ static heat_status profile_arm(Engine* e, double* d_delta, std::vector<double>& 
 }
 
 static heat_status profile_check(Engine* e) {
-  if (e->ks.loop) {
+  if (e->ks.loop || e->has_res) {
     CUDA_TRY(cudaMemcpy(e->h_abort, &e->d_sync->abort, sizeof(int), cudaMemcpyDeviceToHost));
     if (*e->h_abort) {
       heat_status st = loop_abort(e);
@@ -1068,7 +1343,33 @@ heat_status engine_profile(Engine* e, int reps, void* flush, size_t flush_bytes,
     cudaGetLastError();
     st = set_error(HEAT_ERR_NOMEM, "profile: no room for the residual norms");
   }
-  for (int done = 0; done < reps && st == HEAT_OK;) {
+  const bool on_chip = e->has_res && !e->has_stream;
+  for (int done = 0; done < reps && st == HEAT_OK && on_chip;) {
+    // one launch runs a chunk of iterations; its time per iteration is reported as the apply's
+    const int c = std::min(reps - done, chunk);
+    st = loop_sync_reset(e, c);
+    if (st == HEAT_OK) st = profile_arm(e, d_delta, h_delta);
+    if (st != HEAT_OK) break;
+    if (flush) k_flush_read<<<sm_count() * 4, 256, 0, e->stream>>>((const uint4*)flush, flush_bytes / 16, (unsigned int*)e->d_unfinished);
+    cudaEventRecord(ev[0], e->stream);
+    cudaError_t le = res_launch(e, e->stream);
+    cudaEventRecord(ev[1], e->stream);
+    if (le != cudaSuccess || cudaStreamSynchronize(e->stream) != cudaSuccess) {
+      cudaGetLastError();
+      st = set_error(HEAT_ERR_CUDA, "profile: launch failed");
+      break;
+    }
+    float a = 0.f;
+    cudaEventElapsedTime(&a, ev[0], ev[1]);
+    ta += a;
+    st = profile_check(e);
+    done += c;
+  }
+  if (on_chip) {
+    const heat_status st2 = loop_sync_reset(e);
+    if (st == HEAT_OK) st = st2;
+  }
+  for (int done = 0; done < reps && st == HEAT_OK && !on_chip;) {
     const int c = std::min(reps - done, chunk);
     st = profile_arm(e, d_delta, h_delta);
     if (st != HEAT_OK) break;
@@ -1123,8 +1424,8 @@ heat_status engine_profile(Engine* e, int reps, void* flush, size_t flush_bytes,
       bu += n * (2 * 4 + 4 + 2 * 4 + 4 + 4);
     }
   }
-  *bytes_apply = ba;
-  *bytes_update = bu;
+  *bytes_apply = on_chip ? ba + bu : ba;
+  *bytes_update = on_chip ? 0.0 : bu;
   return HEAT_OK;
 }
 
@@ -1149,9 +1450,10 @@ heat_status engine_time_iterations(Engine* e, int reps, double* ms_per_iter) {
   // 40 iterations per timed chunk: below the inner cap, and on small meshes
   // short of the point where a seeded residual has converged to rounding
   constexpr int kChunk = 40;
-  const int per_tick = e->ks.loop ? kChunk : e->iters_per_tick;
-  const int chunk_ticks = e->ks.loop ? 1 : std::max(1, kChunk / e->iters_per_tick);
-  if (e->ks.loop) {
+  const bool persistent = e->ks.loop || (e->has_res && !e->has_stream);
+  const int per_tick = persistent ? kChunk : e->iters_per_tick;
+  const int chunk_ticks = persistent ? 1 : std::max(1, kChunk / e->iters_per_tick);
+  if (persistent) {
     heat_status st = loop_sync_reset(e, kChunk);
     if (st != HEAT_OK) return st;
   }
@@ -1193,7 +1495,7 @@ heat_status engine_time_iterations(Engine* e, int reps, double* ms_per_iter) {
   cudaEventDestroy(a);
   cudaEventDestroy(b);
   cudaFree(d_delta);
-  if (e->ks.loop) {
+  if (persistent) {
     const heat_status st2 = loop_sync_reset(e);
     if (st == HEAT_OK) st = st2;
   }
@@ -1230,7 +1532,7 @@ static std::vector<int> wave_segments(heat_sim* const* sims, int nsims, int prec
     long long items = 0;
     for (int i = 0; i < nsims; ++i) {
       SimDev d = sims[i]->dev;
-      tile_geometry(d, k2);
+      tile_geometry(d, k2, prec == P_FP64);
       items += d.w_items;
     }
     const long long waves = (items + cap - 1) / cap;
@@ -1259,7 +1561,8 @@ heat_status engine_autotune(heat_sim* const* sims, int nsims, int reps, int* bes
   std::vector<double> vbest(kNumVariants, 1e300);
   for (int v = -1; v < kNumVariants && st == HEAT_OK; ++v) {
     if (v >= 0 && prec == P_FP64 && !kVariants[v].f64[0]) continue;
-    for (int si = 0; si < (v < 0 ? 1 : 4) && st == HEAT_OK; ++si) {
+    // the on-chip solve does not depend on the segment size
+    for (int si = 0; si < (v < 0 || kVariants[v].res ? 1 : 4) && st == HEAT_OK; ++si) {
       Tuning t = base;
       t.variant[prec] = v;
       if (v >= 0) t.seg_nodes[bucket] = kSegs[si];

@@ -22,6 +22,10 @@ using LoopFn = void (*)(const SimDev*, const int2*, const int2*, const int*, Gri
 // Its instance for a register-prefetch warp-apply shape (segment width, rows,
 // warps) and pointwise item size (groups per thread); nullptr if none.
 LoopFn loop_kernel(int sx, int ny, int warps, int qpt);
+// The on-chip inner solve (res_kernels.cuh): sims, each block's range of
+// tasks, tasks (simulation, box), wait state.
+using ResFn = void (*)(const SimDev*, const int*, const int2*, GridSync*);
+ResFn res_kernel(bool fp64, int elem);
 }
 
 struct heat_sim {

@@ -73,6 +73,13 @@ struct SimScalars {
   long long steps_total;
 };
 
+// The on-chip inner solve (res_kernels.cuh): the mesh cut into g = gx*gy*gz
+// boxes of at most bx x by x bz nodes, one per block; zc levels per march tile.
+struct ResGeo {
+  int g;  // blocks of this simulation (0: the streaming kernels iterate it)
+  int gx, gy, gz, bx, by, bz, zc;
+};
+
 struct alignas(16) SimDev {  // 16-byte aligned: blocks copy it with uint4 loads
   int nx, ny, nz;             // elements per dimension
   int ntx, nty, ntz, ntiles;  // operator tiles (x, y, z counts and total)
@@ -153,6 +160,14 @@ struct alignas(16) SimDev {  // 16-byte aligned: blocks copy it with uint4 loads
   double* partial;            // 2 per tile
   int* iters_log;             // CG iterations of each step
   int iters_log_len;
+  ResGeo res;
+  // on-chip solve: exchanged boundary values (one tagged word group per
+  // node, rows padded to 4), per-block x and P^-1, the blocks' tagged partial
+  // sums (two sets of g + 1) and the last tag used
+  unsigned char* res_z;
+  unsigned char* res_x;
+  ulonglong2* res_slots;
+  unsigned int* res_tag;
   SimScalars* sc;
 };
 

@@ -296,34 +296,45 @@ struct AsyncSrc {
   __device__ __forceinline__ void after_elements(const LaneGeo<NY>&, int, int) {}
 };
 
+// The march's constants for the operator (sa M + sb K): with lam_q and lam'_q
+// = lam_{q+4} (the two z-Walsh indices of an xy index q), the face sum and the
+// element's top half are
+//   G_q = Tp_q + A_q Fp_q + B_q F_q,  Tn_q = B_q Fp_q + A_q F_q,
+//   A_q = lam_q + lam'_q,  B_q = lam_q - lam'_q,
+// and A_q, B_q are linear in (rho_c, k) with these coefficients. The four
+// xy indices are processed as two pairs, h = 0: q = (0, 1), h = 1: q = (2, 3).
+template <class T>
+struct MarchQ1 {
+  using V = Pair2<T>;
+  using T2 = typename V::t;
+  T2 AM[2], AK[2], BM[2], BK[2];
+  MarchQ1() = default;
+  __device__ __forceinline__ MarchQ1(const SimDev& s, T sa, T sb) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int q0 = 2 * h, q1 = 2 * h + 1;
+      AM[h] = V::make(sa * (lam_m<T>(s, q0) + lam_m<T>(s, q0 + 4)), sa * (lam_m<T>(s, q1) + lam_m<T>(s, q1 + 4)));
+      AK[h] = V::make(sb * (lam_k<T>(s, q0) + lam_k<T>(s, q0 + 4)), sb * (lam_k<T>(s, q1) + lam_k<T>(s, q1 + 4)));
+      BM[h] = V::make(sa * (lam_m<T>(s, q0) - lam_m<T>(s, q0 + 4)), sa * (lam_m<T>(s, q1) - lam_m<T>(s, q1 + 4)));
+      BK[h] = V::make(sb * (lam_k<T>(s, q0) - lam_k<T>(s, q0 + 4)), sb * (lam_k<T>(s, q1) - lam_k<T>(s, q1 + 4)));
+    }
+  }
+};
+
 // Every lane of the segment must call this with the same tzl (the trip count
 // of the level loop): shuffles span the segment. Segments with no tile pass
 // active = false (they load and store nothing). Levels beyond the mesh are
 // zero; outputs are clipped to the mesh. out(node, dirichlet, y, v) receives
 // the operator output y and the node's own input value v.
 template <class T, int SX, int NY, class Src, class Out>
-__device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const SimDev& s, Src& src, int tzl, T sa,
-                                                T sb, Out&& out) {
+__device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MarchQ1<T>& mc, Src& src, int tzl,
+                                                Out&& out) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NR = NY + 2;  // staged rows
   constexpr int NF = NY + 1;  // faces / element rows
-  // With lam_q and lam'_q = lam_{q+4} (the two z-Walsh indices of an xy index
-  // q), the face sum and the element's top half are
-  //   G_q = Tp_q + A_q Fp_q + B_q F_q,  Tn_q = B_q Fp_q + A_q F_q,
-  //   A_q = lam_q + lam'_q,  B_q = lam_q - lam'_q,
-  // and A_q, B_q are linear in (rho_c, k) with these coefficients. The four
-  // xy indices are processed as two pairs, h = 0: q = (0, 1), h = 1: q = (2, 3).
   using V = Pair2<T>;
   using T2 = typename V::t;
-  T2 AM[2], AK[2], BM[2], BK[2];
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int q0 = 2 * h, q1 = 2 * h + 1;
-    AM[h] = V::make(sa * (lam_m<T>(s, q0) + lam_m<T>(s, q0 + 4)), sa * (lam_m<T>(s, q1) + lam_m<T>(s, q1 + 4)));
-    AK[h] = V::make(sb * (lam_k<T>(s, q0) + lam_k<T>(s, q0 + 4)), sb * (lam_k<T>(s, q1) + lam_k<T>(s, q1 + 4)));
-    BM[h] = V::make(sa * (lam_m<T>(s, q0) - lam_m<T>(s, q0 + 4)), sa * (lam_m<T>(s, q1) - lam_m<T>(s, q1 + 4)));
-    BK[h] = V::make(sb * (lam_k<T>(s, q0) - lam_k<T>(s, q0 + 4)), sb * (lam_k<T>(s, q1) - lam_k<T>(s, q1 + 4)));
-  }
+  const T2 (&AM)[2] = mc.AM, (&AK)[2] = mc.AK, (&BM)[2] = mc.BM, (&BK)[2] = mc.BK;
   const T2 M1 = V::make(T(-1), T(-1));  // a - b = fma(b, M1, a), exact as a subtraction
   src.prologue(lg, tzl);
   T2 Fp[NF][2], Tp[NF][2];
@@ -414,14 +425,23 @@ __device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const Sim
 // <= 8 boxes' contributions in a fixed order: the upper corners of the layer
 // below (carried in registers), then this layer's lower corners, the left
 // neighbour's through one shuffle per row.
+template <class T>
+struct MarchP1 {
+  T mw, kwx, kwy, kwz;  // sa V / 20 and sb V / h_a^2, V = hx hy hz / 6
+  MarchP1() = default;
+  __device__ __forceinline__ MarchP1(const SimDev& s, T sa, T sb)
+      : mw(sa * p1_consts<T>(s)[0]),
+        kwx(sb * p1_consts<T>(s)[1]),
+        kwy(sb * p1_consts<T>(s)[2]),
+        kwz(sb * p1_consts<T>(s)[3]) {}
+};
 template <class T, int SX, int NY, class Src, class Out>
-__device__ __forceinline__ void warp_tile_march_p1(const LaneGeo<NY>& lg, const SimDev& s, Src& src, int tzl, T sa,
-                                                   T sb, Out&& out) {
+__device__ __forceinline__ void warp_tile_march_p1(const LaneGeo<NY>& lg, const MarchP1<T>& mc, Src& src, int tzl,
+                                                   Out&& out) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NR = NY + 2;  // staged rows
   constexpr int NF = NY + 1;  // box rows
-  const T mw = sa * p1_consts<T>(s)[0];  // V / 20 and V / h_a^2, V = hx hy hz / 6
-  const T kwx = sb * p1_consts<T>(s)[1], kwy = sb * p1_consts<T>(s)[2], kwz = sb * p1_consts<T>(s)[3];
+  const T mw = mc.mw, kwx = mc.kwx, kwy = mc.kwy, kwz = mc.kwz;
   src.prologue(lg, tzl);
   T prv[NR], prvR[NR], carry[NY];
 #pragma unroll
@@ -488,14 +508,21 @@ __device__ __forceinline__ void warp_tile_march_p1(const LaneGeo<NY>& lg, const 
   }
 }
 
-// The march of element type E.
+// The march of element type E and its constants.
+template <int E, class T>
+using MarchE = typename std::conditional<E == E_P1, MarchP1<T>, MarchQ1<T>>::type;
+template <int E, class T, int SX, int NY, class Src, class Out>
+__device__ __forceinline__ void warp_march_c(const LaneGeo<NY>& lg, const MarchE<E, T>& mc, Src& src, int tzl,
+                                             Out&& out) {
+  if constexpr (E == E_P1)
+    warp_tile_march_p1<T, SX, NY>(lg, mc, src, tzl, out);
+  else
+    warp_tile_march<T, SX, NY>(lg, mc, src, tzl, out);
+}
 template <int E, class T, int SX, int NY, class Src, class Out>
 __device__ __forceinline__ void warp_march_e(const LaneGeo<NY>& lg, const SimDev& s, Src& src, int tzl, T sa, T sb,
                                              Out&& out) {
-  if constexpr (E == E_P1)
-    warp_tile_march_p1<T, SX, NY>(lg, s, src, tzl, sa, sb, out);
-  else
-    warp_tile_march<T, SX, NY>(lg, s, src, tzl, sa, sb, out);
+  warp_march_c<E, T, SX, NY>(lg, MarchE<E, T>(s, sa, sb), src, tzl, out);
 }
 
 // The register-prefetch form with functor loads (see RegSrc), for element E.

@@ -507,7 +507,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_open_w(const SimDev* __res
         PreRegSrc<TO, NY, typename std::remove_reference<decltype(fetch)>::type,
                   typename std::remove_reference<decltype(value)>::type>
             src(s.acoef, fetch, value, tz * s.o_tz);
-        warp_tile_march<TO, SX, NY>(lg, s, src, s.o_tz, TO(s.inv_dt), TO(s.theta), out);
+        warp_tile_march<TO, SX, NY>(lg, MarchQ1<TO>(s, TO(s.inv_dt), TO(s.theta)), src, s.o_tz, out);
         return;
       }
       op(TO(s.inv_dt), TO(s.theta), mask, fetch, value, out);
