@@ -350,6 +350,10 @@ extern "C" heat_status heat_sim_create(const heat_mesh* mesh, const heat_bc* bc,
     for (int t = 0; t < 4; ++t) d.p1c_f[t] = (float)d.p1c[t];
   }
   walsh_eigenvalues(hx, hy, hz, d.lam_m, d.lam_k);
+  d.sigma[0] = 12.0 / (hx * hx);
+  d.sigma[1] = 12.0 / (hy * hy);
+  d.sigma[2] = 12.0 / (hz * hz);
+  d.m43 = 4.0 / 3.0 * d.lam_m[0];
   for (int p = 0; p < 8; ++p) {
     d.mhat_f[p] = (float)d.mhat[p];
     d.khat_f[p] = (float)d.khat[p];
@@ -769,27 +773,73 @@ extern "C" heat_status heat_step_iterations(heat_sim* s, int step, int* iters) {
 
 // ------------------------------------------------------ operator entry points
 
-extern "C" heat_status heat_apply(heat_sim* s, const double* x, double* y) {
-  if (!s || !x || !y) return set_error(HEAT_ERR_ARG, "heat_apply: null argument");
-  k_apply_nodes<double, true><<<grid_for(s->nn, 128), 128, 0, s->stream>>>(s->d_dev, s->dev.inv_dt, s->dev.theta, x, y);
+// Tiles of the operator entry points (k_op_march), ny rows each: the levels
+// per tile with the least estimated time on sms SMs of occ resident blocks. A
+// tile of tz levels computes tz + 1 element layers and takes about 1.5 more
+// to start; share: the part of an SM's throughput that one block uses (FP64:
+// all of it, though alone on an SM it reaches about 0.8 of that). *time: the estimate in level times of one row.
+static OpTiles op_tiles(const heat_sim* s, int ny, int sms, int occ, double share, double* time) {
+  OpTiles t{};
+  const int levels = s->dev.nz + 1;
+  t.ntx = (s->dev.nx + 1 + 29) / 30;
+  t.nty = (s->dev.ny + 1 + ny - 1) / ny;
+  const long long cols = (long long)t.ntx * t.nty;
+  double best = 1e300;
+  for (int tz = std::min(levels, 64); tz >= 1; --tz) {
+    const long long tiles = cols * ((levels + tz - 1) / tz);
+    const long long b = ((tiles + kOpWarps - 1) / kOpWarps + sms - 1) / sms;  // blocks per SM
+    const double e = (tz + 2.5) * std::max(b == 1 ? 1.25 : (double)((b + occ - 1) / occ), share * (double)b) * (ny + 1);
+    if (e < best * (1.0 - 1e-9)) {
+      best = e;
+      t.tz = tz;
+      t.ntiles = (int)tiles;
+    }
+  }
+  *time = best;
+  return t;
+}
+
+template <class T, int MODE>
+static heat_status op_launch(heat_sim* s, T sa, T sb, const T* x, T* y, int n_step) {
+  int dev = 0, sms = 148;
+  CUDA_TRY(cudaGetDevice(&dev));
+  CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  constexpr bool F64 = sizeof(T) == 8;
+  const bool p1 = s->dev.elem == E_P1;
+  // four rows per lane do the least work, one row spreads a small mesh over
+  // more schedulers (FP64: a warp's instruction takes its scheduler 64 cycles)
+  double e4 = 0.0, e1 = 0.0;
+  const OpTiles t4 = op_tiles(s, 4, sms, F64 ? 2 : 4, F64 ? 1.0 : 0.3, &e4);
+  const OpTiles t1 = op_tiles(s, 1, sms, F64 ? 3 : 6, F64 ? 1.0 : 0.3, &e1);
+  const bool four = e4 <= e1;
+  const OpTiles& t = four ? t4 : t1;
+  const unsigned blocks = (unsigned)((t.ntiles + kOpWarps - 1) / kOpWarps);
+  auto run = [&](auto fn) { fn<<<blocks, 32 * kOpWarps, 0, s->stream>>>(s->d_dev, sa, sb, x, y, n_step, t); };
+  if (four) {
+    if (p1) run(k_op_march<T, 4, MODE, E_P1>);
+    else run(k_op_march<T, 4, MODE, E_Q1>);
+  } else {
+    if (p1) run(k_op_march<T, 1, MODE, E_P1>);
+    else run(k_op_march<T, 1, MODE, E_Q1>);
+  }
   CUDA_TRY(cudaGetLastError());
   return HEAT_OK;
 }
 
+extern "C" heat_status heat_apply(heat_sim* s, const double* x, double* y) {
+  if (!s || !x || !y) return set_error(HEAT_ERR_ARG, "heat_apply: null argument");
+  return op_launch<double, OP_A>(s, s->dev.inv_dt, s->dev.theta, x, y, 0);
+}
+
 extern "C" heat_status heat_apply_f32(heat_sim* s, const float* x, float* y) {
   if (!s || !x || !y) return set_error(HEAT_ERR_ARG, "heat_apply_f32: null argument");
-  k_apply_nodes<float, true><<<grid_for(s->nn, 128), 128, 0, s->stream>>>(s->d_dev, (float)s->dev.inv_dt,
-                                                                          (float)s->dev.theta, x, y);
-  CUDA_TRY(cudaGetLastError());
-  return HEAT_OK;
+  return op_launch<float, OP_A>(s, (float)s->dev.inv_dt, (float)s->dev.theta, x, y, 0);
 }
 
 extern "C" heat_status heat_apply_general(heat_sim* s, double sa, double sb, const double* x, double* y) {
   if (!s || !x || !y) return set_error(HEAT_ERR_ARG, "heat_apply_general: null argument");
   if (!std::isfinite(sa) || !std::isfinite(sb)) return set_error(HEAT_ERR_NONFINITE, "heat_apply_general: scale");
-  k_apply_nodes<double, false><<<grid_for(s->nn, 128), 128, 0, s->stream>>>(s->d_dev, sa, sb, x, y);
-  CUDA_TRY(cudaGetLastError());
-  return HEAT_OK;
+  return op_launch<double, OP_GENERAL>(s, sa, sb, x, y, 0);
 }
 
 extern "C" heat_status heat_diagonal(heat_sim* s, double* p) {
@@ -801,9 +851,7 @@ extern "C" heat_status heat_diagonal(heat_sim* s, double* p) {
 
 extern "C" heat_status heat_rhs(heat_sim* s, int n, const double* u_prev, double* b) {
   if (!s || !u_prev || !b || n < 1) return set_error(HEAT_ERR_ARG, "heat_rhs: bad argument");
-  k_rhs_nodes<<<grid_for(s->nn, 128), 128, 0, s->stream>>>(s->d_dev, n, u_prev, b);
-  CUDA_TRY(cudaGetLastError());
-  return HEAT_OK;
+  return op_launch<double, OP_RHS>(s, s->dev.inv_dt, s->dev.theta - 1.0, u_prev, b, n);
 }
 
 extern "C" heat_status heat_flux_vector(heat_sim* s, double* f) {

@@ -89,7 +89,7 @@ struct alignas(16) SimDev {  // 16-byte aligned: blocks copy it with uint4 loads
   int w_ntx, w_nty, w_ntz, w_tz, w_ntiles;
   int w_items;                // work items (groups of segment tiles per block)
   int fused;                  // the engine runs the FP32 inner solve as one fused kernel per iteration
-  int w_pad_;
+  int w_sx;                   // their segment width (16 or 32 lanes)
   // warp-segment tiles of the step-start and refinement passes (k_open_w):
   // (SX-2) x NY x o_tz nodes each, o_items work items
   int o_ntx, o_nty, o_ntz, o_tz, o_ntiles, o_items;
@@ -111,6 +111,9 @@ struct alignas(16) SimDev {  // 16-byte aligned: blocks copy it with uint4 loads
   // lam_k[w] = sum_d (w_d ? 2/h_d : 0) prod_{d' != d} (...) / 8.
   double lam_m[8], lam_k[8];
   float lam_m_f[8], lam_k_f[8];
+  // lam_w = lam_m[0] 3^-|w| (rho_c + k sum of sigma over w's differences) per
+  // unit scale: sigma[d] = 12 / h_d^2; m43 = 4/3 lam_m[0] (op_warp.cuh)
+  double sigma[3], m43;
   const double2* coef;        // (rho_c, k) per element
   const float2* coef32;
   double* vec64[4];           // U^{n-1}, U^{n-2}, x and spare (slots in SimScalars)

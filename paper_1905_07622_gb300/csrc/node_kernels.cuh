@@ -4,6 +4,7 @@
 #pragma once
 
 #include "op.cuh"
+#include "op_warp.cuh"
 
 namespace heat {
 
@@ -236,44 +237,49 @@ __global__ void k_reciprocal(const double* __restrict__ a, double* __restrict__ 
     out[i] = 1.0 / a[i];
 }
 
-// y = (sa M + sb K) x; with MASK, Dirichlet rows give y = x and Dirichlet
-// columns are dropped (the eliminated operator padded with the identity).
-template <class T, bool MASK>
-__global__ void k_apply_nodes(const SimDev* __restrict__ sp, T sa, T sb, const T* __restrict__ x,
-                              T* __restrict__ y) {
-  const SimDev& s = *sp;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < s.nn;
-       n += (long long)gridDim.x * blockDim.x) {
-    int i, j, k;
-    node_of(s, n, i, j, k);
-    if (MASK && is_dirichlet(s, i, j, k)) {
-      y[n] = x[n];
-      continue;
-    }
-    y[n] = gather_apply<T>(s, sa, sb, i, j, k, [&](int a, int b, int c) -> T {
-      if (MASK && is_dirichlet(s, a, b, c)) return T(0);
-      return x[node_index(s, a, b, c)];
-    });
-  }
-}
+// The operator entry points in the warp-segment march (op_warp.cuh): one
+// 32-lane segment tile of 30 x NY x tz nodes per warp. A node's product once
+// per element corner (one thread per node gathering 8 elements x 8 corners)
+// takes 190 operations and 27 loads; the march about 55 and 1.5.
+//   OP_A: y = A' x, the eliminated operator padded with the identity
+//   OP_GENERAL: y = (sa M + sb K) x, no elimination
+//   OP_RHS: b = L u + F^n - z on free rows, g on Dirichlet rows
+// Measured (one GB300, gathered -> marched): FP32 A' x on 200^3 778 -> 55 us
+// (130 MB, 2.4 TB/s), FP64 right-hand side on 100^3 385 -> 172 us (bound by the
+// FP64 pipe), FP64 A' x on 33x21x17 18.4 -> 12.3 us (one wave of short tiles).
+enum OpMode : int { OP_A = 0, OP_GENERAL = 1, OP_RHS = 2 };
+struct OpTiles {
+  int ntx, nty, ntiles, tz;
+};
+constexpr int kOpWarps = 4;
 
-// Right-hand side of step n from u_prev: b = L u_prev + F^n - z (free rows), g (Dirichlet).
-__global__ void k_rhs_nodes(const SimDev* __restrict__ sp, int n_step, const double* __restrict__ u,
-                            double* __restrict__ b) {
+template <class T, int NY, int MODE, int E>
+__global__ void __launch_bounds__(32 * kOpWarps, sizeof(T) == 8 ? 2 : 4)
+    k_op_march(const SimDev* __restrict__ sp, T sa, T sb, const T* __restrict__ x, T* __restrict__ y, int n_step,
+               OpTiles t) {
   const SimDev& s = *sp;
-  const bool flux_on = s.flux_steps < 0 || n_step <= s.flux_steps;
-  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < s.nn;
-       n += (long long)gridDim.x * blockDim.x) {
-    int i, j, k;
-    node_of(s, n, i, j, k);
-    if (is_dirichlet(s, i, j, k)) {
-      b[n] = dirichlet_value(s, i, j, k);
-      continue;
-    }
-    const double lu = gather_apply<double>(s, s.inv_dt, s.theta - 1.0, i, j, k,
-                                           [&](int a, int bb, int c) -> double { return u[node_index(s, a, bb, c)]; });
-    b[n] = lu + (flux_on ? s.F[n] : 0.0) - s.zlift[n];
-  }
+  const Geo g(s);
+  const int tile = blockIdx.x * kOpWarps + (int)(threadIdx.x >> 5);
+  const bool active = tile < t.ntiles;
+  const int tx = tile % t.ntx, rem = tile / t.ntx, ty = rem % t.nty, tz = rem / t.nty;
+  const bool flux_on = MODE == OP_RHS && (s.flux_steps < 0 || n_step <= s.flux_steps);
+  warp_tile_op_e<E, T, 32, NY>(
+      g, s, coef_ptr<T>(s), active, tx * 30, ty * NY, tz * t.tz, t.tz, sa, sb, MODE == OP_A,
+      [&](int m, bool live) -> T { return live ? x[m] : T(0); }, [](T v) { return v; },
+      [&](int m, bool dir, T yv, T) {
+        if constexpr (MODE == OP_A) {
+          y[m] = dir ? x[m] : yv;
+        } else if constexpr (MODE == OP_GENERAL) {
+          y[m] = yv;
+        } else {
+          if (dir) {
+            const int kk = m / g.pxy, r = m - kk * g.pxy, jj = r / g.px;
+            y[m] = dirichlet_value(s, r - jj * g.px, jj, kk);
+          } else {
+            y[m] = yv + (flux_on ? s.F[m] : 0.0) - s.zlift[m];
+          }
+        }
+      });
 }
 
 // Overwrite Dirichlet nodes of u with their values.

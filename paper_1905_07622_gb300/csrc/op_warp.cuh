@@ -196,6 +196,75 @@ struct RegSrc {
   }
 };
 
+// RegSrc with each element row's coefficients read as a PreRec
+// from SimDev::acoef: the warp-segment march of the A operator with its
+// per-element coefficients precomputed.
+// AHEAD: the coefficients too are loaded one layer ahead into registers; without
+// it each row's are loaded where they are used (FP64: 16 registers per row
+// saved, and the FP64 pipe hides the latency).
+template <class T, int NY, class Fetch, class Value, bool AHEAD = true>
+struct PreRegSrc {
+  static constexpr int NR = NY + 2, NF = NY + 1;
+  using Raw = decltype(std::declval<Fetch&>()(0, false));
+  const float4* __restrict__ pre;
+  Fetch& fetch;
+  Value& value;
+  int k0;
+  Raw raw[NR];
+  PreRec cf[AHEAD ? NF : 1];
+  const LaneGeo<NY>* geo = nullptr;
+
+  __device__ __forceinline__ PreRegSrc(const float4* p, Fetch& f, Value& v, int k0_)
+      : pre(p), fetch(f), value(v), k0(k0_) {}
+  __device__ __forceinline__ void load_nodes(const LaneGeo<NY>& lg, int L) {
+    const unsigned lv = lg.live_rows(L);
+    const int off = lg.nbase + L * lg.pxy;
+#pragma unroll
+    for (int r = 0; r < NR; ++r) {
+      const int m = off + r * lg.px;
+      raw[r] = fetch(m, ((lv >> r) & 1u) && HEAT_INDEX_OK(lg.sc, m, lg.nn));
+    }
+  }
+  __device__ __forceinline__ PreRec load_row(const LaneGeo<NY>& lg, unsigned le, int E, int r) const {
+    PreRec c;
+    const int e = lg.ebase + r * lg.enx + E * lg.estride;
+    if (((le >> r) & 1u) && HEAT_INDEX_OK(lg.sc, e, lg.ne)) {
+      const float4* p = pre + 4 * (long long)e;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) c.w[w] = __ldg(p + w);
+    } else {
+#pragma unroll
+      for (int w = 0; w < 4; ++w) c.w[w] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    return c;
+  }
+  __device__ __forceinline__ void load_coef(const LaneGeo<NY>& lg, int E) {
+    if constexpr (AHEAD) {
+      const unsigned le = lg.live_elems(E);
+#pragma unroll
+      for (int r = 0; r < NF; ++r) cf[r] = load_row(lg, le, E, r);
+    }
+  }
+  __device__ __forceinline__ void prologue(const LaneGeo<NY>& lg, int) {
+    geo = &lg;
+    load_nodes(lg, k0 - 1);
+    load_coef(lg, k0 - 1);
+  }
+  __device__ __forceinline__ void level(const LaneGeo<NY>& lg, int t, int tzl, T v[NR]) {
+#pragma unroll
+    for (int r = 0; r < NR; ++r) v[r] = value(raw[r]);
+    if (t <= tzl) load_nodes(lg, k0 + t);
+  }
+  // element layer k0-2+t
+  __device__ __forceinline__ PreRec coef_row(int t, int r) const {
+    if constexpr (AHEAD) return cf[r];
+    else return load_row(*geo, geo->live_elems(k0 - 2 + t), k0 - 2 + t, r);
+  }
+  __device__ __forceinline__ void after_elements(const LaneGeo<NY>& lg, int t, int tzl) {
+    if (t <= tzl) load_coef(lg, k0 - 1 + t);
+  }
+};
+
 // cp.async of 4, 8 or 16 bytes into shared memory; live = false writes zeros
 // and reads nothing (the source address must still be a valid pointer).
 template <int BYTES>
@@ -301,15 +370,26 @@ struct AsyncSrc {
 // element's top half are
 //   G_q = Tp_q + A_q Fp_q + B_q F_q,  Tn_q = B_q Fp_q + A_q F_q,
 //   A_q = lam_q + lam'_q,  B_q = lam_q - lam'_q,
-// and A_q, B_q are linear in (rho_c, k) with these coefficients. The four
-// xy indices are processed as two pairs, h = 0: q = (0, 1), h = 1: q = (2, 3).
+// and A_q, B_q are linear in (rho_c, k). The four xy indices are processed as
+// two pairs, h = 0: q = (0, 1), h = 1: q = (2, 3).
+//
+// THIRD (float and double coefficients (rho_c, k)): the eigenvalues are
+//   lam_w = m0 3^-|w| (sa rho_c + sb k sigma_w), sigma_w = sum of 12 / h_d^2 over w's differences,
+// so with the factors 1/3 of x and y moved into the inverse butterflies (an
+// addition becomes a multiply-add) the coefficients are A_q = R + K al_q,
+// B_q = R / 2 + K be_q with R = (4/3) m0 sa rho_c, K = m0 sb k: 8 multiply-adds
+// and 3 products per element instead of 16 and 8. Double-float has no
+// multiply-add to hide the 1/3 in and keeps the plain form, as do coefficients
+// that are precomputed (PreRec).
+template <class T, bool THIRD>
+struct MarchQ1T;
 template <class T>
-struct MarchQ1 {
+struct MarchQ1T<T, false> {
   using V = Pair2<T>;
   using T2 = typename V::t;
   T2 AM[2], AK[2], BM[2], BK[2];
-  MarchQ1() = default;
-  __device__ __forceinline__ MarchQ1(const SimDev& s, T sa, T sb) {
+  MarchQ1T() = default;
+  __device__ __forceinline__ MarchQ1T(const SimDev& s, T sa, T sb) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int q0 = 2 * h, q1 = 2 * h + 1;
@@ -319,22 +399,68 @@ struct MarchQ1 {
       BK[h] = V::make(sb * (lam_k<T>(s, q0) - lam_k<T>(s, q0 + 4)), sb * (lam_k<T>(s, q1) - lam_k<T>(s, q1 + 4)));
     }
   }
+  template <class C>
+  __device__ __forceinline__ void coeffs(const C& cf, T2 (&A)[2], T2 (&B)[2]) const {
+    march_coeffs<T>(cf, AM, AK, BM, BK, A, B);
+  }
 };
+template <class T>
+struct MarchQ1T<T, true> {
+  using V = Pair2<T>;
+  using T2 = typename V::t;
+  T2 al[2], be[2];
+  T ra, ka;
+  MarchQ1T() = default;
+  __device__ __forceinline__ MarchQ1T(const SimDev& s, T sa, T sb) {
+    const T third = T(1.0 / 3.0), sz = (T)s.sigma[2];
+    const T sg[4] = {T(0), (T)s.sigma[0], (T)s.sigma[1], (T)s.sigma[0] + (T)s.sigma[1]};
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      al[h] = V::make(third * (T(4) * sg[2 * h] + sz), third * (T(4) * sg[2 * h + 1] + sz));
+      be[h] = V::make(third * (T(2) * sg[2 * h] - sz), third * (T(2) * sg[2 * h + 1] - sz));
+    }
+    ra = (T)s.m43 * sa;
+    ka = lam_m<T>(s, 0) * sb;
+  }
+  template <class C>
+  __device__ __forceinline__ void coeffs(const C& cf, T2 (&A)[2], T2 (&B)[2]) const {
+    const T R = ra * cf.x, K = ka * cf.y, H = T(0.5) * R;
+    const T2 R2 = V::make(R, R), K2 = V::make(K, K), H2 = V::make(H, H);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      A[h] = V::fma(K2, al[h], R2);
+      B[h] = V::fma(K2, be[h], H2);
+    }
+  }
+};
+template <class T>
+using MarchQ1 = MarchQ1T<T, !std::is_same<T, DF>::value>;
+// with precomputed coefficients nothing is needed
+template <class T>
+struct MarchPre {
+  using V = Pair2<T>;
+  using T2 = typename V::t;
+  __device__ __forceinline__ void coeffs(const PreRec& cf, T2 (&A)[2], T2 (&B)[2]) const {
+    const T2 z[2] = {};
+    march_coeffs<T>(cf, z, z, z, z, A, B);
+  }
+};
+template <class MC> struct IsThird : std::false_type {};
+template <class T> struct IsThird<MarchQ1T<T, true>> : std::true_type {};
 
 // Every lane of the segment must call this with the same tzl (the trip count
 // of the level loop): shuffles span the segment. Segments with no tile pass
 // active = false (they load and store nothing). Levels beyond the mesh are
 // zero; outputs are clipped to the mesh. out(node, dirichlet, y, v) receives
 // the operator output y and the node's own input value v.
-template <class T, int SX, int NY, class Src, class Out>
-__device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MarchQ1<T>& mc, Src& src, int tzl,
-                                                Out&& out) {
+template <class T, int SX, int NY, class MC, class Src, class Out>
+__device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC& mc, Src& src, int tzl, Out&& out) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NR = NY + 2;  // staged rows
   constexpr int NF = NY + 1;  // faces / element rows
   using V = Pair2<T>;
   using T2 = typename V::t;
-  const T2 (&AM)[2] = mc.AM, (&AK)[2] = mc.AK, (&BM)[2] = mc.BM, (&BK)[2] = mc.BK;
+  constexpr bool THIRD = IsThird<MC>::value;
   const T2 M1 = V::make(T(-1), T(-1));  // a - b = fma(b, M1, a), exact as a subtraction
   src.prologue(lg, tzl);
   T2 Fp[NF][2], Tp[NF][2];
@@ -374,7 +500,7 @@ __device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const Mar
 #pragma unroll
       for (int r = 0; r < NF; ++r) {
         T2 A[2], B[2];
-        march_coeffs<T>(src.coef_row(t, r), AM, AK, BM, BK, A, B);
+        mc.coeffs(src.coef_row(t, r), A, B);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           G[r][h] = V::fma(B[h], F[r][h], V::fma(A[h], Fp[r][h], Tp[r][h]));
@@ -390,8 +516,19 @@ __device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const Mar
 #pragma unroll
         for (int r = 1; r <= NY; ++r) {
           // (g0, g1) = (G_0 + G_2, G_1 + G_3) of row r + (G_0 - G_2, G_1 - G_3) of row r-1
-          const T2 g = V::add(V::add(G[r][0], G[r][1]), V::fma(G[r - 1][1], M1, G[r - 1][0]));
-          const T nl = g.x + g.y, nr = g.x - g.y;
+          T2 g;
+          T nl, nr;
+          if constexpr (THIRD) {
+            const T2 TH = V::make(T(1.0 / 3.0), T(1.0 / 3.0));
+            // G_0 + G_2 / 3 of row r, G_0 - G_2 / 3 of row r - 1: the thirds of both in one product
+            g = V::fma(V::fma(G[r - 1][1], M1, G[r][1]), TH, V::add(G[r][0], G[r - 1][0]));
+            nl = g.x + T(1.0 / 3.0) * g.y;
+            nr = g.x - T(1.0 / 3.0) * g.y;
+          } else {
+            g = V::add(V::add(G[r][0], G[r][1]), V::fma(G[r - 1][1], M1, G[r - 1][0]));
+            nl = g.x + g.y;
+            nr = g.x - g.y;
+          }
           const T from_left = __shfl_up_sync(FULL, nr, 1, SX);
           const int m = lg.nbase + r * lg.px + lv * lg.pxy;
           if (lg.out_lane && lvin && ((lg.rin >> r) & 1u) && HEAT_INDEX_OK(lg.sc, m, lg.nn)) {

@@ -51,61 +51,6 @@ template <> struct PreAB<DF> {
   }
 };
 
-// RegSrc (op_warp.cuh) with each element row's coefficients read as a PreRec
-// from SimDev::acoef: the warp-segment march of the A operator with its
-// per-element coefficients precomputed.
-template <class T, int NY, class Fetch, class Value>
-struct PreRegSrc {
-  static constexpr int NR = NY + 2, NF = NY + 1;
-  using Raw = decltype(std::declval<Fetch&>()(0, false));
-  const float4* __restrict__ pre;
-  Fetch& fetch;
-  Value& value;
-  int k0;
-  Raw raw[NR];
-  PreRec cf[NF];
-
-  __device__ __forceinline__ PreRegSrc(const float4* p, Fetch& f, Value& v, int k0_)
-      : pre(p), fetch(f), value(v), k0(k0_) {}
-  __device__ __forceinline__ void load_nodes(const LaneGeo<NY>& lg, int L) {
-    const unsigned lv = lg.live_rows(L);
-    const int off = lg.nbase + L * lg.pxy;
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const int m = off + r * lg.px;
-      raw[r] = fetch(m, ((lv >> r) & 1u) && HEAT_INDEX_OK(lg.sc, m, lg.nn));
-    }
-  }
-  __device__ __forceinline__ void load_coef(const LaneGeo<NY>& lg, int E) {
-    const unsigned le = lg.live_elems(E);
-#pragma unroll
-    for (int r = 0; r < NF; ++r) {
-      const int e = lg.ebase + r * lg.enx + E * lg.estride;
-      if (((le >> r) & 1u) && HEAT_INDEX_OK(lg.sc, e, lg.ne)) {
-        const float4* p = pre + 4 * (long long)e;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) cf[r].w[w] = __ldg(p + w);
-      } else {
-#pragma unroll
-        for (int w = 0; w < 4; ++w) cf[r].w[w] = make_float4(0.f, 0.f, 0.f, 0.f);
-      }
-    }
-  }
-  __device__ __forceinline__ void prologue(const LaneGeo<NY>& lg, int) {
-    load_nodes(lg, k0 - 1);
-    load_coef(lg, k0 - 1);
-  }
-  __device__ __forceinline__ void level(const LaneGeo<NY>& lg, int t, int tzl, T v[NR]) {
-#pragma unroll
-    for (int r = 0; r < NR; ++r) v[r] = value(raw[r]);
-    if (t <= tzl) load_nodes(lg, k0 + t);
-  }
-  __device__ __forceinline__ const PreRec& coef_row(int, int r) const { return cf[r]; }
-  __device__ __forceinline__ void after_elements(const LaneGeo<NY>& lg, int t, int tzl) {
-    if (t <= tzl) load_coef(lg, k0 - 1 + t);
-  }
-};
-
 // tile_op (op.cuh) for the A operator on trilinear boxes, with each element's
 // coefficients A_q, B_q read from SimDev::acoef instead of formed from
 // (rho_c, k): the same factorised product and the same contract, about a
@@ -507,7 +452,7 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_open_w(const SimDev* __res
         PreRegSrc<TO, NY, typename std::remove_reference<decltype(fetch)>::type,
                   typename std::remove_reference<decltype(value)>::type>
             src(s.acoef, fetch, value, tz * s.o_tz);
-        warp_tile_march<TO, SX, NY>(lg, MarchQ1<TO>(s, TO(s.inv_dt), TO(s.theta)), src, s.o_tz, out);
+        warp_tile_march<TO, SX, NY>(lg, MarchPre<TO>(), src, s.o_tz, out);
         return;
       }
       op(TO(s.inv_dt), TO(s.theta), mask, fetch, value, out);

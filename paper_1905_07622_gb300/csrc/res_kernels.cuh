@@ -239,6 +239,11 @@ __device__ __forceinline__ bool res_all_sum(const S& v, ulonglong2* mail, int g,
   res_split(v, va, vb);
   const unsigned long long wa = tagged(va, tag), wb = tagged(vb, tag);
   for (int u = lane; u < g; u += 32) st_word2(reinterpret_cast<unsigned long long*>(mail + u * (g + 1) + rank), wa, wb);
+  // A few stores linger on their way for about 4,000 cycles unless something
+  // pushes them: with one store instruction or two a fence is cheaper (21
+  // blocks: 21,100 -> 18,400 cycles an iteration), with more it only costs
+  // (144 blocks: 26,000 -> 27,100).
+  if (g <= 48) __threadfence();
   const unsigned long long* w = reinterpret_cast<const unsigned long long*>(mail + rank * (g + 1));
   const int n = g + (int)gs->extra;
   S t = S(0);
@@ -596,16 +601,13 @@ struct ResQ1 {
   float al[4], be[4];
   float ra, ka;  // R = ra rho_c, K = ka k
   __device__ __forceinline__ void set(const SimDev& s) {
-    const double m0 = s.lam_m[0];
-    // sigma of one difference: lam_k / lam_m of that Walsh index
-    const double sx = s.lam_k[1] / s.lam_m[1], sy = s.lam_k[2] / s.lam_m[2], sz = s.lam_k[4] / s.lam_m[4];
-    const double sg[4] = {0.0, sx, sy, sx + sy};
+    const double sz = s.sigma[2], sg[4] = {0.0, s.sigma[0], s.sigma[1], s.sigma[0] + s.sigma[1]};
     for (int q = 0; q < 4; ++q) {
       al[q] = (float)((4.0 * sg[q] + sz) / 3.0);
       be[q] = (float)((2.0 * sg[q] - sz) / 3.0);
     }
-    ra = (float)(4.0 / 3.0 * m0 * s.inv_dt);
-    ka = (float)(m0 * s.theta);
+    ra = (float)(s.m43 * s.inv_dt);
+    ka = (float)(s.lam_m[0] * s.theta);
   }
 };
 __device__ __forceinline__ float2 res_march(const ResTile& t, const ResQ1& mc, int tzl) {
