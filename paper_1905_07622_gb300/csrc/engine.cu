@@ -43,10 +43,11 @@ struct KernelSet {
   // `open` when set), on their own segment geometry and work list
   TileFn open_w = nullptr;
   int owsx = 0, owny = 0, owwarps = 0;
-  long long open_cap = 0;  // blocks of open_w resident on the GPU at once (0: unknown)
+  int w_occ = 0, o_occ = 0;  // blocks of apply_w and open_w resident on an SM (0: unknown)
   // the CG iterations of a tick as one persistent kernel (replaces the
   // apply and update launches when set; FP32 paths, register-prefetch apply)
   LoopFn loop = nullptr;
+  bool dual = false;  // apply_w takes 16- and 32-lane segments, chosen per mesh (wsx for Chebyshev members)
   // the inner solve held on the chip: iterates the members whose mesh fits
   // (SimDev::res.g > 0); the others take apply and update
   ResFn res = nullptr;
@@ -139,6 +140,8 @@ template <int SX, int NY, int W, int MINB>
 static constexpr WVariant wv_res() {
   WVariant v = wv<SX, NY, W, 0, MINB, 0>();
   v.res = true;
+  v.f32[0] = k_apply_dot_w2<float, NY, W, MINB, E_Q1>;
+  v.f32[1] = k_apply_dot_w2<float, NY, W, MINB, E_P1>;
   return v;
 }
 // (segment width, rows, warps, stages, min blocks per SM for float / double,
@@ -155,7 +158,8 @@ constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
 // variant per precision (-1: the block-tile apply) and the segment tile size
 // per mesh-size bucket. Both are fixed per simulation size, so results stay
 // bitwise identical alone and in batches built under the same table.
-static Tuning g_tuning = {{-1, 0, 0}, {512, 512, 512}, {2, 4, 4}, {2, 2, 2}, {0, 0, 0}};
+constexpr int kAutoSeg = 512;  // the default segment size: levels per tile from pick_levels
+static Tuning g_tuning = {{-1, 0, 0}, {kAutoSeg, kAutoSeg, kAutoSeg}, {2, 4, 4}, {2, 2, 2}, {0, 0, 0}};
 static std::mutex g_tuning_mu;
 
 int num_variants() { return kNumVariants; }
@@ -250,10 +254,10 @@ static int res_nodes(const ResGeo& r) { return r.bx * r.by * r.bz; }
 // Estimated cycles of one iteration on boxes r, fitted to clock readings in
 // the kernel (boxes of 16^3 to 105^3 meshes): a march layer takes a warp 850
 // cycles alone on its scheduler and 690 beside others, a pointwise group of
-// 4 nodes per thread 640 over the passes, an all-sum about 3,000 with its
+// 4 nodes per thread 640 over the passes, an all-sum about 4,000 with its
 // block barriers.
 static double res_cycles(const ResGeo& r, bool fp64) {
-  const double sums = r.g > 1 ? 6200.0 + 5.0 * r.g : 2600.0;
+  const double sums = r.g > 1 ? 7600.0 + 5.0 * r.g : 2100.0;
   if (fp64) {
     // a warp's FP64 instruction takes its scheduler 64 cycles; 27 + 6 of them per node and iteration
     const int warps = (res_nodes(r) + 31) / 32;
@@ -347,6 +351,16 @@ static ResBytes res_bytes(const SimDev& d, bool fp64) {
   return b;
 }
 
+// Blocks of a kernel resident on an SM (0: unknown, as without a GPU).
+static int occupancy(TileFn fn, int threads, int smem) {
+  int occ = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, threads, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return occ;
+}
+
 // The kernels of precision prec under tuning table t. With Chebyshev passes
 // (cheb) a fused variant is replaced by the register-prefetch variant of the
 // same segment shape: the fused iteration has no place for the passes.
@@ -387,21 +401,34 @@ static KernelSet kernel_set(int prec, const Tuning& t, bool cheb = false, int el
       // prefetch, separate update, no Chebyshev passes
       if (t.loop[prec] && prec != P_FP64 && elem == E_Q1 && !cheb && !v.fused && !v.res && v.stages == 0)
         k.loop = loop_kernel(v.sx, v.ny, v.warps, t.pw_quads[prec]);
-      if (v.res) res_kernel_set(k, false, elem);
+      if (v.res) {
+        res_kernel_set(k, false, elem);
+        k.dual = true;
+      }
     }
   }
-  if (prec == P_FP64 && variant < 0) res_kernel_set(k, true, elem);
+  if (prec == P_FP64 && variant < 0) {
+    // FP64 by default: on the chip where the mesh fits; else 16-lane segments
+    // of 4 rows (the FP64 pipe bounds the apply, and 4 rows compute 5 rows'
+    // elements where 2 compute 3)
+    res_kernel_set(k, true, elem);
+    // One block of 8 warps per SM: with two smaller ones, blocks that start
+    // early (programmatic launch) pile up two to an SM while others stay empty
+    // (100^3: 23.0 ms a step against 19.1 with the block tiles).
+    k.apply_w = ei ? k_apply_dot_w<double, 16, 4, 8, 0, 1, E_P1> : k_apply_dot_w<double, 16, 4, 8, 0, 1, E_Q1>;
+    k.wsx = 16;
+    k.wny = 4;
+    k.wwarps = 8;
+    k.cheb_w = ei ? k_cheb_w<double, 16, 4, 8, 1, E_P1> : k_cheb_w<double, 16, 4, 8, 1, E_Q1>;
+  }
   if (elem == E_Q1 && t.open_w[prec]) {
     k.open_w = open_w_kernel(prec, t.open_w[prec]);
     k.owsx = kOpenSX;
     k.owny = open_w_rows(t.open_w[prec]);
     k.owwarps = kOpenWarps;
-    int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k.open_w, 32 * kOpenWarps, 0) == cudaSuccess && occ > 0)
-      k.open_cap = (long long)sm_count() * occ;
-    else
-      cudaGetLastError();
+    k.o_occ = occupancy(k.open_w, 32 * kOpenWarps, 0);
   }
+  if (k.apply_w) k.w_occ = occupancy(k.apply_w, 32 * k.wwarps, k.apply_w_smem);
   for (int b = 0; b < 3; ++b) k.seg_nodes[b] = t.seg_nodes[b];
   const int qpt = t.pw_quads[prec];
   k.pw_chunk = pw_chunk(qpt);
@@ -561,6 +588,33 @@ static int members_ncheb(const Engine* e) { return members_ncheb_of(e->sims.data
 // and with them the order of every reduction, are the same whether the
 // simulation runs alone or in a batch: its results are bitwise identical.
 constexpr long long kTileNodes = 2048;
+
+// Levels per segment tile for `cols` segment columns of `levels` node levels,
+// spc tiles per block, at most hi levels. A block with tz levels takes
+// tz + 2.5 level times (halo layers and start); an SM with b blocks takes
+// ceil(b / occ) of those, or b * share where one block alone uses that share
+// of the SM's throughput (1 where the FP64 pipe bounds the kernel: a second
+// block then only waits for the first). The least time^weight * work wins:
+// weight 1 for a launch whose time alone counts as much as the work it adds
+// to a batch, less where the launch is a part of many batched ones. It
+// depends on the mesh and the GPU only, so a simulation's tiles, and with
+// them the order of its reductions, are the same alone and in a batch.
+static int pick_levels(long long cols, int levels, int spc, int occ, double share, double weight, int hi) {
+  const int sms = sm_count();
+  double best = 1e300;
+  int best_tz = std::min(levels, hi);
+  for (int tz = std::min(levels, hi); tz >= 1; --tz) {
+    const long long ntz = (levels + tz - 1) / tz, items = (cols * ntz + spc - 1) / spc, b = (items + sms - 1) / sms;
+    const double t = (tz + 2.5) * std::max((double)((b + occ - 1) / occ), share * (double)b);
+    const double cost = std::pow(t, weight) * (double)ntz * (tz + 2.5);
+    if (cost < best * (1.0 - 1e-9)) {
+      best = cost;
+      best_tz = tz;
+    }
+  }
+  return best_tz;
+}
+
 static void tile_geometry(SimDev& d, const KernelSet& ks, bool fp64) {
   d.res = res_plan(d, ks, fp64);
   d.ntx = (d.nx + 1 + ks.sx - 2) / (ks.sx - 1);
@@ -576,45 +630,33 @@ static void tile_geometry(SimDev& d, const KernelSet& ks, bool fp64) {
   d.npw = (int)((d.nn + ks.pw_chunk - 1) / ks.pw_chunk);
   d.w_ntx = d.w_nty = d.w_ntz = d.w_tz = d.w_ntiles = d.w_items = 0;
   if (ks.apply_w) {
-    // segment tiles of about seg output nodes, at least 4 levels (2 extra levels per tile)
+    // segment tiles of about seg output nodes, at least 4 levels (2 extra levels
+    // per tile); the default size stands for the estimated best
     const int seg = ks.seg_nodes[size_bucket(d.nn)];
-    d.w_ntx = (d.nx + 1 + ks.wsx - 3) / (ks.wsx - 2);
+    // the narrower padded row; equal: whole lines
+    const int pad16 = (d.nx + 1 + 13) / 14 * 14, pad32 = (d.nx + 1 + 29) / 30 * 30;
+    d.w_sx = ks.dual && d.cheb_m < 2 ? (pad32 <= pad16 ? 32 : 16) : ks.wsx;
+    d.w_ntx = (d.nx + 1 + d.w_sx - 3) / (d.w_sx - 2);
     d.w_nty = (d.ny + 1 + ks.wny - 1) / ks.wny;
-    const int tz0 = std::max(4, std::min(levels, seg / ((ks.wsx - 2) * ks.wny)));
+    const int spc = ks.wwarps * (32 / d.w_sx);
+    const int tz0 = seg == kAutoSeg && ks.w_occ > 0
+                        ? pick_levels((long long)d.w_ntx * d.w_nty, levels, spc, ks.w_occ, fp64 ? 1.0 : 0.34, 4.0, 96)
+                        : std::max(4, std::min(levels, seg / ((d.w_sx - 2) * ks.wny)));
     d.w_ntz = (levels + tz0 - 1) / tz0;
     d.w_tz = (levels + d.w_ntz - 1) / d.w_ntz;
     d.w_ntiles = d.w_ntx * d.w_nty * d.w_ntz;
-    const int spc = ks.wwarps * (32 / ks.wsx);
     d.w_items = (d.w_ntiles + spc - 1) / spc;
   }
   d.o_ntx = d.o_nty = d.o_ntz = d.o_tz = d.o_ntiles = d.o_items = 0;
   if (ks.open_w) {
-    // about kOpenSegNodes output nodes per segment tile, at least 4 levels
-    constexpr int kOpenSegNodes = 1024;
     d.o_ntx = (d.nx + 1 + ks.owsx - 3) / (ks.owsx - 2);
     d.o_nty = (d.ny + 1 + ks.owny - 1) / ks.owny;
-    const long long cols = (long long)d.o_ntx * d.o_nty;
     const int spc = ks.owwarps * (32 / ks.owsx);
-    const int tz_def = std::max(4, std::min(levels, kOpenSegNodes / ((ks.owsx - 2) * ks.owny)));
-    auto items_for = [&](int tz) { return (cols * ((levels + tz - 1) / tz) + spc - 1) / spc; };
-    int tz0 = tz_def;
-    // A mesh whose passes fill at least half of the resident blocks in at
-    // most two waves takes the tile height in [tz_def / 2, tz_def] whose
-    // items fill the waves best (the 100^3 mesh: 404 items of 26 levels on
-    // 456 resident blocks instead of 303 of 34). It depends on the mesh and
-    // the GPU only, so a simulation's passes stay the same alone and in a batch.
-    const long long cap = ks.open_cap, items_def = items_for(tz_def);
-    if (cap > 0 && 2 * items_def >= cap && items_def <= 2 * cap) {
-      double best = -1.0;
-      for (int tz = tz_def; tz >= std::max(4, tz_def / 2); --tz) {
-        const long long it = items_for(tz), waves = (it + cap - 1) / cap;
-        const double eff = (double)it / (double)(waves * cap);
-        if (eff > best + 1e-12) {
-          best = eff;
-          tz0 = tz;
-        }
-      }
-    }
+    // at most about 1,024 output nodes per segment tile
+    const int hi = std::max(4, 1024 / ((ks.owsx - 2) * ks.owny));
+    const int tz0 = ks.o_occ > 0 ? pick_levels((long long)d.o_ntx * d.o_nty, levels, spc, ks.o_occ, fp64 ? 1.0 : 0.34,
+                                                 fp64 ? 1.0 : 0.25, hi)
+                                 : std::min(levels, hi);
     d.o_ntz = (levels + tz0 - 1) / tz0;
     d.o_tz = (levels + d.o_ntz - 1) / d.o_ntz;
     d.o_ntiles = d.o_ntx * d.o_nty * d.o_ntz;

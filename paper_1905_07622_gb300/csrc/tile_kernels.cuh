@@ -381,7 +381,19 @@ __device__ __forceinline__ void apply_w_item(const SimDev& s, const Ctl& c, int 
     dnew[m] = v;
     acc += v * qv;
   };
-  if constexpr (STAGES == 0) {
+  if constexpr (STAGES == 0 && sizeof(T) == 8 && E == E_Q1) {
+    // FP64: each element's A_q, B_q are read (64 bytes, SimDev::acoef) instead
+    // of formed. The FP64 pipe bounds this kernel (a warp's instruction takes
+    // its scheduler 64 cycles), and forming them is a third of its operations.
+    const LaneGeo<NY> lg(g, active, (int)threadIdx.x % SX, SX, tx * (SX - 2), ty * NY, true, s.sc);
+    auto fetch = [&](int m, bool live) -> DirRaw<T> {
+      if (!live) return {T(0), T(0), T(0)};
+      return {pinv[m], r[m], rs ? T(0) : dold[m]};
+    };
+    auto value = [&](const DirRaw<T>& v) -> T { return v.p * v.r + beta * v.d; };
+    PreRegSrc<T, NY, decltype(fetch), decltype(value), false> src(s.acoef, fetch, value, tz * s.w_tz);
+    warp_tile_march<T, SX, NY>(lg, MarchPre<T>(), src, s.w_tz, out);
+  } else if constexpr (STAGES == 0) {
     warp_tile_op_e<E, T, SX, NY>(
         g, s, IterVecs<T>::coef(s), active, tx * (SX - 2), ty * NY, tz * s.w_tz, s.w_tz, (T)s.inv_dt,
         (T)s.theta, true,
@@ -436,6 +448,28 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_apply_dot_w(const SimDev* 
     cache_sim(sims, wi.x, cache, cur, dep);
     if (cache.c.phase != PH_ITER) continue;
     apply_w_item<T, SX, NY, WARPS, STAGES, E, false>(cache.s, cache.c, wi.y, red, stage_smem);
+  }
+}
+
+// k_apply_dot_w with the segment width chosen per simulation (SimDev::w_sx):
+// 32-lane segments read whole 128-byte lines (200^3: 66.5 us against 74.6),
+// 16-lane ones fit a row of nodes more closely (120^3: 22.9 us against 24.4).
+template <class T, int NY, int WARPS, int MINB, int E = E_Q1>
+__global__ void __launch_bounds__(32 * WARPS, MINB) k_apply_dot_w2(const SimDev* __restrict__ sims,
+                                                             const int2* __restrict__ work,
+                                                             const int* __restrict__ nwork_p) {
+  __shared__ double red[32];
+  __shared__ ItemCache cache;
+  int cur = -1;
+  bool dep = false;
+  allow_next_launch();
+  const int nwork = *nwork_p;
+  for (int w = blockIdx.x; w < nwork; w += gridDim.x) {
+    const int2 wi = work[w];
+    cache_sim(sims, wi.x, cache, cur, dep);
+    if (cache.c.phase != PH_ITER) continue;
+    if (cache.s.w_sx == 32) apply_w_item<T, 32, NY, WARPS, 0, E, false>(cache.s, cache.c, wi.y, red, nullptr);
+    else apply_w_item<T, 16, NY, WARPS, 0, E, false>(cache.s, cache.c, wi.y, red, nullptr);
   }
 }
 
