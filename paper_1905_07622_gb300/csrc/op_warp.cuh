@@ -35,6 +35,8 @@ template <> struct Pair2<float> {
   static __device__ __forceinline__ float2 add(float2 a, float2 b) { return __fadd2_rn(a, b); }
   static __device__ __forceinline__ float2 mul(float2 a, float2 b) { return __fmul2_rn(a, b); }
   static __device__ __forceinline__ float2 fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+  // a - b, exact as a subtraction
+  static __device__ __forceinline__ float2 sub(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 };
 template <> struct Pair2<double> {
   using t = double2;
@@ -44,6 +46,7 @@ template <> struct Pair2<double> {
   static __device__ __forceinline__ double2 fma(double2 a, double2 b, double2 c) {
     return make_double2(::fma(a.x, b.x, c.x), ::fma(a.y, b.y, c.y));
   }
+  static __device__ __forceinline__ double2 sub(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
 };
 
 // Double-float pairs (df.cuh): the refinement passes' arithmetic, about 48
@@ -54,6 +57,7 @@ template <> struct Pair2<DF> {
   static __device__ __forceinline__ DF2 add(DF2 a, DF2 b) { return DF2{a.x + b.x, a.y + b.y}; }
   static __device__ __forceinline__ DF2 mul(DF2 a, DF2 b) { return DF2{a.x * b.x, a.y * b.y}; }
   static __device__ __forceinline__ DF2 fma(DF2 a, DF2 b, DF2 c) { return DF2{a.x * b.x + c.x, a.y * b.y + c.y}; }
+  static __device__ __forceinline__ DF2 sub(DF2 a, DF2 b) { return DF2{a.x - b.x, a.y - b.y}; }
 };
 
 // One element's precomputed Walsh-pair coefficients A_0..A_3, B_0..B_3 of the
@@ -453,15 +457,19 @@ template <class T> struct IsThird<MarchQ1T<T, true>> : std::true_type {};
 // active = false (they load and store nothing). Levels beyond the mesh are
 // zero; outputs are clipped to the mesh. out(node, dirichlet, y, v) receives
 // the operator output y and the node's own input value v.
-template <class T, int SX, int NY, class MC, class Src, class Out>
-__device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC& mc, Src& src, int tzl, Out&& out) {
+//
+// pre(node, in) loads what out needs at a node (in false: nothing to load, no
+// output); it runs before a level's arithmetic and out receives its result,
+// so those loads are in flight meanwhile.
+template <class T, int SX, int NY, class MC, class Src, class Pre, class Out>
+__device__ __forceinline__ void warp_tile_march_pre(const LaneGeo<NY>& lg, const MC& mc, Src& src, int tzl, Pre&& pre,
+                                                    Out&& out) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NR = NY + 2;  // staged rows
   constexpr int NF = NY + 1;  // faces / element rows
   using V = Pair2<T>;
   using T2 = typename V::t;
   constexpr bool THIRD = IsThird<MC>::value;
-  const T2 M1 = V::make(T(-1), T(-1));  // a - b = fma(b, M1, a), exact as a subtraction
   src.prologue(lg, tzl);
   T2 Fp[NF][2], Tp[NF][2];
   T vprev[NY];
@@ -480,6 +488,13 @@ __device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC&
     const int L = k0 - 1 + t;
     T v[NR];
     src.level(lg, t, tzl, v);
+    decltype(pre(0, false)) got[NY];
+#pragma unroll
+    for (int r = 1; r <= NY; ++r) {
+      const int m = lg.nbase + r * lg.px + (L - 1) * lg.pxy;
+      got[r - 1] = pre(m, t >= 2 && lg.out_lane && L - 1 <= lg.gnz && ((lg.rin >> r) & 1u) != 0u &&
+                              HEAT_INDEX_OK(lg.sc, m, lg.nn));
+    }
     // forward x (edges of each row, as the pair (sum, difference)) and
     // forward y (faces between rows): F[r][0] = (F_0, F_1), F[r][1] = (F_2, F_3)
     T2 E[NR];
@@ -492,7 +507,7 @@ __device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC&
 #pragma unroll
     for (int r = 0; r < NF; ++r) {
       F[r][0] = V::add(E[r], E[r + 1]);
-      F[r][1] = V::fma(E[r + 1], M1, E[r]);
+      F[r][1] = V::sub(E[r], E[r + 1]);
     }
     if (t >= 1) {
       // elements (c, j0-1+r, L-1) between face levels L-1 and L
@@ -521,11 +536,11 @@ __device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC&
           if constexpr (THIRD) {
             const T2 TH = V::make(T(1.0 / 3.0), T(1.0 / 3.0));
             // G_0 + G_2 / 3 of row r, G_0 - G_2 / 3 of row r - 1: the thirds of both in one product
-            g = V::fma(V::fma(G[r - 1][1], M1, G[r][1]), TH, V::add(G[r][0], G[r - 1][0]));
+            g = V::fma(V::sub(G[r][1], G[r - 1][1]), TH, V::add(G[r][0], G[r - 1][0]));
             nl = g.x + T(1.0 / 3.0) * g.y;
             nr = g.x - T(1.0 / 3.0) * g.y;
           } else {
-            g = V::add(V::add(G[r][0], G[r][1]), V::fma(G[r - 1][1], M1, G[r - 1][0]));
+            g = V::add(V::add(G[r][0], G[r][1]), V::sub(G[r - 1][0], G[r - 1][1]));
             nl = g.x + g.y;
             nr = g.x - g.y;
           }
@@ -533,7 +548,7 @@ __device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC&
           const int m = lg.nbase + r * lg.px + lv * lg.pxy;
           if (lg.out_lane && lvin && ((lg.rin >> r) & 1u) && HEAT_INDEX_OK(lg.sc, m, lg.nn)) {
             const bool dir = ((lg.rdxy >> r) & 1u) || dzl;
-            out(m, dir, nl + from_left, vprev[r - 1]);
+            out(m, dir, nl + from_left, vprev[r - 1], got[r - 1]);
           }
         }
       }
@@ -545,6 +560,13 @@ __device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC&
 #pragma unroll
       for (int h = 0; h < 2; ++h) Fp[r][h] = F[r][h];
   }
+}
+
+struct NoPre {};
+template <class T, int SX, int NY, class MC, class Src, class Out>
+__device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC& mc, Src& src, int tzl, Out&& out) {
+  warp_tile_march_pre<T, SX, NY>(lg, mc, src, tzl, [](int, bool) { return NoPre{}; },
+                                 [&](int m, bool dir, T y, T v, NoPre) { out(m, dir, y, v); });
 }
 
 // The same contract on six-tetrahedra boxes (heat.h HEAT_ELEM_P1). Each lane

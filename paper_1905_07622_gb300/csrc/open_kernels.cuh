@@ -15,6 +15,10 @@ namespace heat {
 struct D2 {
   double a, b;
 };
+struct XE {
+  double x;
+  float e;
+};
 
 // Arithmetic of the operator passes of k_open: FP64 on the FP64 path. On the
 // FP32 paths the passes form the refinement's right-hand side and true
@@ -213,9 +217,31 @@ __device__ __forceinline__ void open_passes(const SimDev& s, const Ctl& c, const
     const double* __restrict__ y1 = s.yv[c.iu1];
     const double* __restrict__ y2 = s.yv[c.iu2];
     // pass 1: b = L u^{n-1} + F^n - A_{.D} g (free rows), g (Dirichlet rows)
+    struct At {
+      double f, lift, pinv, u, u2, y, y2;
+      float p32;
+    };
     op(inv_dt, theta_m1, false,
         [&](int m, bool live) -> double { return live ? u1[m] : 0.0; }, ident,
-        [&](int m, bool dir, TO yo, TO) {
+        [&](int m, bool in) -> At {
+          At a{};
+          if (in) {
+            a.f = flux_on ? F[m] : 0.0;
+            a.lift = lift[m];
+            a.pinv = pinv[m];
+            if (use_y) {
+              a.u = u1[m];  // the staged input in FP64
+              a.y = y1[m];
+              a.p32 = s.pinv32[m];
+              if (hp) {
+                a.u2 = u2[m];
+                a.y2 = y2[m];
+              }
+            }
+          }
+          return a;
+        },
+        [&](int m, bool dir, TO yo, TO, const At& a) {
           const double y = to_d(yo);
           if (dir) {
             b[m] = dval(m);
@@ -224,44 +250,58 @@ __device__ __forceinline__ void open_passes(const SimDev& s, const Ctl& c, const
               r32out[m] = 0.f;
             }
           } else {
-            const double bn = y + (flux_on ? F[m] : 0.0) - lift[m];
+            const double bn = y + a.f - a.lift;
             b[m] = bn;
-            part[1] += bn * bn * pinv[m];
+            part[1] += bn * bn * a.pinv;
             if (use_y) {
-              const double v = u1[m];  // the staged input, read back in FP64
-              x[m] = hp ? 2.0 * v - u2[m] : v;
-              const double rn = bn - (hp ? 2.0 * y1[m] - y2[m] : y1[m]);
-              const float r32 = (float)rn;
+              x[m] = hp ? 2.0 * a.u - a.u2 : a.u;
+              const double rn = bn - (hp ? 2.0 * a.y - a.y2 : a.y);
+              const float r32 = df_narrow(rn);
               r32out[m] = r32;
-              acc2 += r32 * r32 * s.pinv32[m];
-              part[0] += rn * rn * pinv[m];
+              acc2 += r32 * r32 * a.p32;
+              part[0] += rn * rn * a.pinv;
             }
           }
         });
     // pass 2: x0 = 2u^{n-1} - u^{n-2} (u^{n-1} on the first step), r = b - A' x0
+    struct At2 {
+      double u, u2, b, pinv;
+      float p32;
+    };
     if (!use_y) opA(true,
         [&](int m, bool live) -> D2 {
           if (!live) return {0.0, 0.0};
           return {u1[m], hp ? u2[m] : u1[m]};
         },
         [](const D2& r) { return 2.0 * r.a - r.b; },
-        [&](int m, bool dir, TO yo, TO) {
+        [&](int m, bool in) -> At2 {
+          At2 a{};
+          if (in) {
+            a.u = u1[m];
+            if (hp) a.u2 = u2[m];
+            a.b = b[m];
+            a.pinv = pinv[m];
+            if (P != P_FP64) a.p32 = s.pinv32[m];
+          }
+          return a;
+        },
+        [&](int m, bool dir, TO yo, TO, const At2& a) {
           const double y = to_d(yo);
           double rn = 0.0;
           if (dir) {
             x[m] = dval(m);
           } else {
-            x[m] = hp ? 2.0 * u1[m] - u2[m] : u1[m];  // the staged input, formed again in FP64
-            rn = b[m] - y;
+            x[m] = hp ? 2.0 * a.u - a.u2 : a.u;  // the staged input, formed again in FP64
+            rn = a.b - y;
           }
           if (P == P_FP64) {
             s.r[m] = rn;
           } else {
-            const float r32 = (float)rn;
+            const float r32 = df_narrow(rn);
             r32out[m] = r32;
-            acc2 += r32 * r32 * s.pinv32[m];
+            acc2 += r32 * r32 * a.p32;
           }
-          part[0] += rn * rn * pinv[m];
+          part[0] += rn * rn * a.pinv;
         });
   } else if (phase == PH_OUTER) {
     // x64 <- x64 + e32 (into the spare slot), r = b - A' x64 in FP64
@@ -269,37 +309,54 @@ __device__ __forceinline__ void open_passes(const SimDev& s, const Ctl& c, const
     double* __restrict__ xa = s.vec64[c.ixa];
     double* __restrict__ ya = s.yv[c.ixa];  // A' x64, used by the next step if this one closes
     const float* __restrict__ e32 = s.e32;
+    struct At {
+      double x, b, pinv;
+      float e, p32;
+    };
     opA(true,
-        [&](int m, bool live) -> D2 {
-          if (!live) return {0.0, 0.0};
-          return {x[m], (double)e32[m]};
+        [&](int m, bool live) -> XE {
+          if (!live) return {0.0, 0.f};
+          return {x[m], e32[m]};
         },
-        [](const D2& r) { return r.a + r.b; },
-        [&](int m, bool dir, TO yo, TO) {
+        [](const XE& r) { return r.x + df_widen(r.e); },
+        [&](int m, bool in) -> At {
+          At a{};
+          if (in) a = {x[m], b[m], pinv[m], e32[m], s.pinv32[m]};
+          return a;
+        },
+        [&](int m, bool dir, TO yo, TO, const At& a) {
           const double y = to_d(yo);
           double rn = 0.0;
           if (dir) {
             xa[m] = dval(m);
           } else {
-            xa[m] = x[m] + (double)e32[m];  // the staged input, formed again in FP64
+            xa[m] = a.x + df_widen(a.e);  // the staged input, formed again in FP64
             ya[m] = y;
-            rn = b[m] - y;
+            rn = a.b - y;
           }
-          const float r32 = (float)rn;
+          const float r32 = df_narrow(rn);
           r32out[m] = r32;
-          acc2 += r32 * r32 * s.pinv32[m];
-          part[0] += rn * rn * pinv[m];
+          acc2 += r32 * r32 * a.p32;
+          part[0] += rn * rn * a.pinv;
         });
   } else {  // PH_RESID (FP64): r = b - A' x, x already advanced by k_update
     const double* __restrict__ x = s.vec64[c.ix];
     double* __restrict__ r = s.r;
+    struct At {
+      double b, pinv;
+    };
     opA(true,
         [&](int m, bool live) -> double { return live ? x[m] : 0.0; }, ident,
-        [&](int m, bool dir, TO yo, TO) {
+        [&](int m, bool in) -> At {
+          At a{};
+          if (in) a = {b[m], pinv[m]};
+          return a;
+        },
+        [&](int m, bool dir, TO yo, TO, const At& a) {
           const double y = to_d(yo);
-          const double rn = dir ? 0.0 : b[m] - y;
+          const double rn = dir ? 0.0 : a.b - y;
           r[m] = rn;
-          part[0] += rn * rn * pinv[m];
+          part[0] += rn * rn * a.pinv;
         });
   }
   part[2] += (double)acc2;
@@ -395,17 +452,19 @@ __global__ void __launch_bounds__(SX* SY) k_open(const SimDev* __restrict__ sims
     const Geo g(s);
     const TileCoords tc = tile_coords<SX, SY>(s, wi.y);
     double part[3] = {0.0, 0.0, 0.0};
-    auto op = [&](TO sa, TO sb, bool mask, auto&& fetch, auto&& value, auto&& out) {
-      tile_op_e<E, TO, SX, SY>(g, s, s.coef, tc.i0, tc.j0, tc.k0, tc.nzt, sa, sb, mask, sh, fetch, value, out);
+    auto op = [&](TO sa, TO sb, bool mask, auto&& fetch, auto&& value, auto&& pre, auto&& out) {
+      tile_op_e<E, TO, SX, SY>(g, s, s.coef, tc.i0, tc.j0, tc.k0, tc.nzt, sa, sb, mask, sh, fetch, value,
+                               [&](int m, bool dir, TO y, TO v) { out(m, dir, y, v, pre(m, true)); });
     };
-    auto opA = [&](bool mask, auto&& fetch, auto&& value, auto&& out) {
+    auto opA = [&](bool mask, auto&& fetch, auto&& value, auto&& pre, auto&& out) {
       if constexpr (E == E_Q1) {
         if (s.acoef) {
-          tile_op_pre<TO, SX, SY>(g, s, tc.i0, tc.j0, tc.k0, tc.nzt, mask, sh, fetch, value, out);
+          tile_op_pre<TO, SX, SY>(g, s, tc.i0, tc.j0, tc.k0, tc.nzt, mask, sh, fetch, value,
+                                  [&](int m, bool dir, TO y, TO v) { out(m, dir, y, v, pre(m, true)); });
           return;
         }
       }
-      op(TO(s.inv_dt), TO(s.theta), mask, fetch, value, out);
+      op(TO(s.inv_dt), TO(s.theta), mask, fetch, value, pre, out);
     };
     open_passes<P>(s, c, g, phase, part, op, opA);
     double tot[3];
@@ -442,20 +501,23 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) k_open_w(const SimDev* __res
     const bool active = tile < s.o_ntiles;
     const int tx = tile % s.o_ntx, rem = tile / s.o_ntx, ty = rem % s.o_nty, tz = rem / s.o_nty;
     double part[3] = {0.0, 0.0, 0.0};
-    auto op = [&](TO sa, TO sb, bool mask, auto&& fetch, auto&& value, auto&& out) {
-      warp_tile_op_e<E_Q1, TO, SX, NY>(g, s, s.coef, active, tx * (SX - 2), ty * NY, tz * s.o_tz, s.o_tz, sa, sb,
-                                       mask, fetch, value, out);
+    const LaneGeo<NY> lg_free(g, active, (int)threadIdx.x % SX, SX, tx * (SX - 2), ty * NY, true, s.sc);
+    const LaneGeo<NY> lg_all(g, active, (int)threadIdx.x % SX, SX, tx * (SX - 2), ty * NY, false, s.sc);
+    auto op = [&](TO sa, TO sb, bool mask, auto&& fetch, auto&& value, auto&& pre, auto&& out) {
+      RegSrc<TO, NY, double2, typename std::remove_reference<decltype(fetch)>::type,
+             typename std::remove_reference<decltype(value)>::type>
+          src(s.coef, fetch, value, tz * s.o_tz);
+      warp_tile_march_pre<TO, SX, NY>(mask ? lg_free : lg_all, MarchQ1<TO>(s, sa, sb), src, s.o_tz, pre, out);
     };
-    auto opA = [&](bool mask, auto&& fetch, auto&& value, auto&& out) {
+    auto opA = [&](bool mask, auto&& fetch, auto&& value, auto&& pre, auto&& out) {
       if (s.acoef) {
-        const LaneGeo<NY> lg(g, active, (int)threadIdx.x % SX, SX, tx * (SX - 2), ty * NY, mask, s.sc);
         PreRegSrc<TO, NY, typename std::remove_reference<decltype(fetch)>::type,
                   typename std::remove_reference<decltype(value)>::type>
             src(s.acoef, fetch, value, tz * s.o_tz);
-        warp_tile_march<TO, SX, NY>(lg, MarchPre<TO>(), src, s.o_tz, out);
+        warp_tile_march_pre<TO, SX, NY>(mask ? lg_free : lg_all, MarchPre<TO>(), src, s.o_tz, pre, out);
         return;
       }
-      op(TO(s.inv_dt), TO(s.theta), mask, fetch, value, out);
+      op(TO(s.inv_dt), TO(s.theta), mask, fetch, value, pre, out);
     };
     open_passes<P>(s, c, g, phase, part, op, opA);
     double tot[3];
