@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(32 * kOpWarps, sizeof(T) == 8 ? 2 : 4)
   const bool flux_on = MODE == OP_RHS && (s.flux_steps < 0 || n_step <= s.flux_steps);
   warp_tile_op_e<E, T, 32, NY>(
       g, s, coef_ptr<T>(s), active, tx * 30, ty * NY, tz * t.tz, t.tz, sa, sb, MODE == OP_A,
-      [&](int m, bool live) -> T { return live ? x[m] : T(0); }, [](T v) { return v; },
+      [&](int m, bool live) -> T { return ld_if(x + m, live); }, [](T v) { return v; },
       [&](int m, bool dir, T yv, T) {
         if constexpr (MODE == OP_A) {
           y[m] = dir ? x[m] : yv;

@@ -148,6 +148,25 @@ struct LaneGeo {
   __device__ __forceinline__ unsigned live_elems(int E) const { return (E >= 0 && E < gnz) ? ein : 0u; }
 };
 
+// *p where live, else zero: one predicated load, no branch around it (FP32;
+// the FP64 kernels wait for the FP64 pipe instead). A time step on 200^3, which
+// streams its vectors: 184.6 -> 180.0 ms.
+__device__ __forceinline__ float ld_if(const float* p, bool live) {
+  float v;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.f32 %0, 0f00000000;\n\t@p ld.global.f32 %0, [%1];\n\t}"
+               : "=f"(v) : "l"(p), "r"((int)live));
+  return v;
+}
+__device__ __forceinline__ float2 ld_if(const float2* p, bool live) {
+  float2 v;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.f32 %0, 0f00000000;\n\tmov.f32 %1, 0f00000000;\n\t"
+               "@p ld.global.v2.f32 {%0, %1}, [%2];\n\t}"
+               : "=f"(v.x), "=f"(v.y) : "l"(p), "r"((int)live));
+  return v;
+}
+__device__ __forceinline__ double ld_if(const double* p, bool live) { return live ? *p : 0.0; }
+__device__ __forceinline__ double2 ld_if(const double2* p, bool live) { return live ? *p : make_double2(0.0, 0.0); }
+
 // Loads one level ahead into registers through caller-supplied functors:
 // fetch(node, live) -> Raw, value(Raw) -> T.
 template <class T, int NY, class Coef, class Fetch, class Value>
@@ -175,11 +194,8 @@ struct RegSrc {
     const unsigned le = lg.live_elems(E);
 #pragma unroll
     for (int r = 0; r < NF; ++r) {
-      Coef z;
-      z.x = 0;
-      z.y = 0;
       const int e = lg.ebase + r * lg.enx + E * lg.estride;
-      cf[r] = (((le >> r) & 1u) && HEAT_INDEX_OK(lg.sc, e, lg.ne)) ? coef[e] : z;
+      cf[r] = ld_if(coef + e, ((le >> r) & 1u) && HEAT_INDEX_OK(lg.sc, e, lg.ne));
     }
   }
   // before the loop: node level k0-1, element layer k0-1 (used at t = 1)
