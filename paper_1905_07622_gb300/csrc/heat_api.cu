@@ -256,21 +256,22 @@ heat_status heat::sim_derive_async(heat_sim* s) {
   const int g = grid_for(s->nn, 256);
   CUDA_TRY(cudaMemsetAsync(&s->d_sc->y_valid, 0, sizeof(int), s->stream));
   CUDA_TRY(cudaMemsetAsync(s->d_bad, 0, sizeof(unsigned int), s->stream));
-  k_setup_coef32<<<grid_for(s->ne, 256), 256, 0, s->stream>>>(s->d_dev, s->ne, s->d_bad);
+  k_setup_coef32<<<grid_for(s->ne, 256), 256, 0, s->stream>>>(s->d_dev, s->ne, s->d_bad, nullptr, nullptr);
   k_setup_diag<<<g, 256, 0, s->stream>>>(s->d_dev);
   k_setup_lift<<<g, 256, 0, s->stream>>>(s->d_dev);
   CUDA_TRY(cudaGetLastError());
   return sim_setup_cheb(s);
 }
 
-static heat_status sim_refresh(heat_sim* s) {
+// rc, kk: device arrays of new coefficients (null: those in place)
+static heat_status sim_refresh(heat_sim* s, const double* rc = nullptr, const double* kk = nullptr) {
   heat_status st = sim_upload_desc(s);
   if (st != HEAT_OK) return st;
   const int g = grid_for(s->nn, 256);
   // the operator changes: stored products A' u of past states no longer hold
   CUDA_TRY(cudaMemsetAsync(&s->d_sc->y_valid, 0, sizeof(int), s->stream));
   CUDA_TRY(cudaMemsetAsync(s->d_bad, 0, sizeof(unsigned int), s->stream));
-  k_setup_coef32<<<grid_for(s->ne, 256), 256, 0, s->stream>>>(s->d_dev, s->ne, s->d_bad);
+  k_setup_coef32<<<grid_for(s->ne, 256), 256, 0, s->stream>>>(s->d_dev, s->ne, s->d_bad, rc, kk);
   k_setup_diag<<<g, 256, 0, s->stream>>>(s->d_dev);
   k_setup_lift<<<g, 256, 0, s->stream>>>(s->d_dev);
   CUDA_TRY(cudaGetLastError());
@@ -484,25 +485,25 @@ extern "C" heat_status heat_set_coeffs(heat_sim* s, const double* rho_c, const d
         return set_error(HEAT_ERR_ARG, "heat_set_coeffs: coefficients must be > 0 (element %lld)", e);
     }
   }
-  // Stage both arrays in the b and q work vectors (Ne < N), check them on the
-  // device, and only then interleave them into the live (rho_c, k) array.
-  const size_t bytes = (size_t)s->ne * sizeof(double);
-  heat_status st = copy_in(s, s->dev.b, rho_c, bytes, on_device);
-  if (st != HEAT_OK) return st;
-  st = copy_in(s, s->dev.q, k, bytes, on_device);
-  if (st != HEAT_OK) return st;
+  // Device arrays are checked before anything live is changed; arrays of the
+  // host, checked above, are staged in the b and q work vectors (Ne < N). The
+  // setup kernel interleaves them into the live (rho_c, k) array.
+  if (!on_device) {
+    const size_t bytes = (size_t)s->ne * sizeof(double);
+    heat_status st = copy_in(s, s->dev.b, rho_c, bytes, 0);
+    if (st != HEAT_OK) return st;
+    st = copy_in(s, s->dev.q, k, bytes, 0);
+    if (st != HEAT_OK) return st;
+    return sim_refresh(s, s->dev.b, s->dev.q);
+  }
   CUDA_TRY(cudaMemsetAsync(s->d_bad, 0, sizeof(unsigned int), s->stream));
-  k_check_coef_pair<<<grid_for(s->ne, 256), 256, 0, s->stream>>>(s->dev.b, s->dev.q, s->ne, s->d_bad);
+  k_check_coef_pair<<<grid_for(s->ne, 256), 256, 0, s->stream>>>(rho_c, k, s->ne, s->d_bad);
   CUDA_TRY(cudaGetLastError());
   unsigned int bad = 0;
   CUDA_TRY(cudaMemcpyAsync(&bad, s->d_bad, sizeof(bad), cudaMemcpyDeviceToHost, s->stream));
   CUDA_TRY(cudaStreamSynchronize(s->stream));
   if (bad) return set_error(HEAT_ERR_NONFINITE, "heat_set_coeffs: %u coefficient(s) non-finite or not > 0", bad);
-  CUDA_TRY(cudaMemcpy2DAsync((void*)s->dev.coef, sizeof(double2), s->dev.b, sizeof(double), sizeof(double),
-                             (size_t)s->ne, cudaMemcpyDeviceToDevice, s->stream));
-  CUDA_TRY(cudaMemcpy2DAsync((char*)s->dev.coef + sizeof(double), sizeof(double2), s->dev.q, sizeof(double),
-                             sizeof(double), (size_t)s->ne, cudaMemcpyDeviceToDevice, s->stream));
-  return sim_refresh(s);
+  return sim_refresh(s, rho_c, k);
 }
 
 extern "C" heat_status heat_get_coeffs(heat_sim* s, double* rho_c, double* k, int on_device) {

@@ -15,6 +15,8 @@ namespace heat {
 // K'_cc of the node's local corner c in each box). Writes 1/P in FP64 and FP32.
 __global__ void k_setup_diag(const SimDev* __restrict__ sp) {
   const SimDev& s = *sp;
+  const bool p1 = s.elem == E_P1;
+  const double inv_dt = s.inv_dt, theta = s.theta, cm = inv_dt * s.mhat[0], ck = theta * s.khat[0];
   for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < s.nn;
        n += (long long)gridDim.x * blockDim.x) {
     int i, j, k;
@@ -22,11 +24,12 @@ __global__ void k_setup_diag(const SimDev* __restrict__ sp) {
     double p = 1.0;
     if (!is_dirichlet(s, i, j, k)) {
       double sa = 0.0, sk = 0.0;
+#pragma unroll
       for (int c = 0; c < 8; ++c) {
         const int ex = i - (c & 1), ey = j - ((c >> 1) & 1), ez = k - ((c >> 2) & 1);
         if (ex < 0 || ey < 0 || ez < 0 || ex >= s.nx || ey >= s.ny || ez >= s.nz) continue;
         const double2 cf = s.coef[ex + (long long)s.nx * (ey + (long long)s.ny * ez)];
-        if (s.elem == E_P1) {
+        if (p1) {
           sa += cf.x * s.p1w[9 * c];
           sk += cf.y * s.p1w[64 + 9 * c];
         } else {
@@ -34,10 +37,11 @@ __global__ void k_setup_diag(const SimDev* __restrict__ sp) {
           sk += cf.y;
         }
       }
-      p = s.elem == E_P1 ? s.inv_dt * sa + s.theta * sk : s.inv_dt * s.mhat[0] * sa + s.theta * s.khat[0] * sk;
+      p = p1 ? inv_dt * sa + theta * sk : cm * sa + ck * sk;
     }
-    s.pinv[n] = 1.0 / p;
-    s.pinv32[n] = (float)(1.0 / p);
+    const double r = 1.0 / p;
+    s.pinv[n] = r;
+    s.pinv32[n] = (float)r;
   }
 }
 
@@ -172,7 +176,13 @@ __global__ void k_setup_lift(const SimDev* __restrict__ sp) {
     int i, j, k;
     node_of(s, n, i, j, k);
     double z = 0.0;
-    if (s.dir_faces && !is_dirichlet(s, i, j, k)) {
+    // a node with a Dirichlet neighbour lies one layer from such a face; every
+    // other node's terms are all zero (200^3 with one face fixed: 2.98 ms when
+    // each node gathered them)
+    const bool near = ((s.dir_faces & 1u) && i == 1) || ((s.dir_faces & 2u) && i == s.nx - 1) ||
+                      ((s.dir_faces & 4u) && j == 1) || ((s.dir_faces & 8u) && j == s.ny - 1) ||
+                      ((s.dir_faces & 16u) && k == 1) || ((s.dir_faces & 32u) && k == s.nz - 1);
+    if (near && !is_dirichlet(s, i, j, k)) {
       z = gather_apply<double>(s, s.inv_dt, s.theta, i, j, k, [&](int a, int b, int c) -> double {
         return is_dirichlet(s, a, b, c) ? dirichlet_value(s, a, b, c) : 0.0;
       });
@@ -181,28 +191,59 @@ __global__ void k_setup_lift(const SimDev* __restrict__ sp) {
   }
 }
 
+// Finite and > 0, from the bits: an FP64 comparison takes a scheduler 64 cycles.
+__device__ __forceinline__ bool positive_finite(double v) {
+  const long long u = __double_as_longlong(v);
+  return u > 0 && u < 0x7ff0000000000000ll;
+}
+
 // FP32 copy of the coefficients; counts non-finite or non-positive entries.
+// With rc, kk the pairs are interleaved from them into SimDev::coef first.
 // On trilinear boxes also the A operator's per-element Walsh-pair
 // coefficients (SimDev::acoef): A_q = rc/dt (lm_q + lm_{q+4}) + theta k
 // (lk_q + lk_{q+4}), B_q the same with differences, computed in FP64 and
 // stored as FP64 (FP64 path) or as (hi, lo) float pairs (FP32 paths).
-__global__ void k_setup_coef32(const SimDev* __restrict__ sp, long long ne, unsigned int* bad) {
+// Bound by the FP64 pipe: the sums of eigenvalues are formed once per thread
+// and the pairs split by integer arithmetic (df.cuh), 20 FP64 instructions an
+// element; with both done per element in FP64 74 us on 80^3, now 41.
+__global__ void k_setup_coef32(const SimDev* __restrict__ sp, long long ne, unsigned int* bad, const double* rc,
+                               const double* kk) {
   const SimDev& s = *sp;
   unsigned int nbad = 0;
+  const bool op = s.acoef && s.elem == E_Q1, f64 = s.prec == P_FP64;
+  double ms[4], md[4], ks[4], kd[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    ms[q] = s.lam_m[q] + s.lam_m[q + 4];
+    md[q] = s.lam_m[q] - s.lam_m[q + 4];
+    ks[q] = s.lam_k[q] + s.lam_k[q + 4];
+    kd[q] = s.lam_k[q] - s.lam_k[q + 4];
+  }
+  const double inv_dt = s.inv_dt, theta = s.theta;
+  double2* __restrict__ coef = const_cast<double2*>(s.coef);
+  float2* __restrict__ coef32 = const_cast<float2*>(s.coef32);
+  float4* __restrict__ acoef = const_cast<float4*>(s.acoef);
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ne;
        e += (long long)gridDim.x * blockDim.x) {
-    const double2 c = s.coef[e];
-    if (!(isfinite(c.x) && isfinite(c.y) && c.x > 0.0 && c.y > 0.0)) ++nbad;
-    reinterpret_cast<float2*>(const_cast<float2*>(s.coef32))[e] = make_float2((float)c.x, (float)c.y);
-    if (s.acoef && s.elem == E_Q1) {
-      const double a = s.inv_dt * c.x, b = s.theta * c.y;
+    double2 c;
+    if (rc) {
+      c = make_double2(rc[e], kk[e]);
+      coef[e] = c;
+    } else {
+      c = coef[e];
+    }
+    if (!positive_finite(c.x) || !positive_finite(c.y)) ++nbad;
+    coef32[e] = make_float2((float)c.x, (float)c.y);
+    if (op) {
+      const double a = inv_dt * c.x, b = theta * c.y;
       double A[4], B[4];
+#pragma unroll
       for (int q = 0; q < 4; ++q) {
-        A[q] = a * (s.lam_m[q] + s.lam_m[q + 4]) + b * (s.lam_k[q] + s.lam_k[q + 4]);
-        B[q] = a * (s.lam_m[q] - s.lam_m[q + 4]) + b * (s.lam_k[q] - s.lam_k[q + 4]);
+        A[q] = a * ms[q] + b * ks[q];
+        B[q] = a * md[q] + b * kd[q];
       }
-      float4* out = const_cast<float4*>(s.acoef) + 4 * e;
-      if (s.prec == P_FP64) {
+      float4* out = acoef + 4 * e;
+      if (f64) {
         double2* o = reinterpret_cast<double2*>(out);
         o[0] = make_double2(A[0], A[1]);
         o[1] = make_double2(A[2], A[3]);
@@ -210,12 +251,12 @@ __global__ void k_setup_coef32(const SimDev* __restrict__ sp, long long ne, unsi
         o[3] = make_double2(B[2], B[3]);
       } else {
         float h[8], l[8];
+#pragma unroll
         for (int q = 0; q < 4; ++q) {
-          h[q] = (float)A[q];
-          l[q] = (float)(A[q] - (double)h[q]);
-          h[q + 4] = (float)B[q];
-          l[q + 4] = (float)(B[q] - (double)h[q + 4]);
+          df_split(A[q], h[q], l[q]);
+          df_split(B[q], h[q + 4], l[q + 4]);
         }
+#pragma unroll
         for (int w = 0; w < 4; ++w) out[w] = make_float4(h[2 * w], l[2 * w], h[2 * w + 1], l[2 * w + 1]);
       }
     }
@@ -228,7 +269,7 @@ __global__ void k_check_coef_pair(const double* __restrict__ rc, const double* _
                                   unsigned int* bad) {
   unsigned int nbad = 0;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ne; e += (long long)gridDim.x * blockDim.x)
-    if (!(isfinite(rc[e]) && isfinite(kk[e]) && rc[e] > 0.0 && kk[e] > 0.0)) ++nbad;
+    if (!positive_finite(rc[e]) || !positive_finite(kk[e])) ++nbad;
   if (nbad) atomicAdd(bad, nbad);
 }
 
