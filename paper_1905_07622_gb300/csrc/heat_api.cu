@@ -364,49 +364,64 @@ extern "C" heat_status heat_sim_create(const heat_mesh* mesh, const heat_bc* bc,
   fill_params(s);
 
   const size_t N8 = (size_t)s->nn * 8, N4 = (size_t)s->nn * 4;
-  void* p;
-#define ALLOC(field, bytes, type)          \
-  st = sim_alloc(s, &p, (bytes));          \
-  if (st != HEAT_OK) goto fail;            \
-  field = (type)p;
-  ALLOC(d.coef, (size_t)s->ne * sizeof(double2), const double2*);
-  ALLOC(d.coef32, (size_t)s->ne * sizeof(float2), const float2*);
-  ALLOC(d.acoef, (size_t)s->ne * 4 * sizeof(float4), const float4*);
-  for (int v = 0; v < 4; ++v) { ALLOC(d.vec64[v], N8, double*); }
-  for (int v = 0; v < 4; ++v) { ALLOC(d.yv[v], N8, double*); }
-  ALLOC(d.b, N8, double*);
-  ALLOC(d.r, N8, double*);
-  ALLOC(d.q, N8, double*);
-  ALLOC(d.d[0], N8, double*);
-  ALLOC(d.d[1], N8, double*);
-  ALLOC(d.pinv, N8, double*);
-  ALLOC(d.zlift, N8, double*);
-  ALLOC(d.F, N8, double*);
-  ALLOC(d.r32, N4, float*);
-  ALLOC(d.q32, N4, float*);
-  ALLOC(d.e32, N4, float*);
-  ALLOC(d.d32[0], N4, float*);
-  ALLOC(d.d32[1], N4, float*);
-  ALLOC(d.pinv32, N4, float*);
-  ALLOC(d.rc32[1], N4, float*);
-  ALLOC(d.wc32[1], N4, float*);
-  ALLOC(d.p32, N4, float*);
-  ALLOC(d.z32, N4, float*);
-  ALLOC(d.cheb, sizeof(double) * 20, double*);
+  // One allocation holds every array: a simulation had 37, and the calls that
+  // made and freed them took longer than a request's set-up (48^3: a create
+  // and destroy 1.7 ms).
+  struct Part {
+    void** field;
+    size_t bytes;
+  };
+  std::vector<Part> parts;
+  auto want = [&](auto& field, size_t bytes) { parts.push_back({(void**)(&field), (bytes + 255) & ~(size_t)255}); };
+  want(d.coef, (size_t)s->ne * sizeof(double2));
+  want(d.coef32, (size_t)s->ne * sizeof(float2));
+  want(d.acoef, (size_t)s->ne * 4 * sizeof(float4));
+  for (int v = 0; v < 4; ++v) want(d.vec64[v], N8);
+  for (int v = 0; v < 4; ++v) want(d.yv[v], N8);
+  want(d.b, N8);
+  want(d.r, N8);
+  want(d.q, N8);
+  want(d.d[0], N8);
+  want(d.d[1], N8);
+  want(d.pinv, N8);
+  want(d.zlift, N8);
+  want(d.F, N8);
+  want(d.r32, N4);
+  want(d.q32, N4);
+  want(d.e32, N4);
+  want(d.d32[0], N4);
+  want(d.d32[1], N4);
+  want(d.pinv32, N4);
+  want(d.rc32[1], N4);
+  want(d.wc32[1], N4);
+  want(d.p32, N4);
+  want(d.z32, N4);
+  want(d.cheb, sizeof(double) * 20);
+  s->iters_log_cap = 4096;
+  want(d.iters_log, sizeof(int) * s->iters_log_cap);
+  d.iters_log_len = s->iters_log_cap;
+  want(s->d_dev, sizeof(SimDev));
+  want(s->d_sc, sizeof(SimScalars));
+  want(s->d_q6, sizeof(double) * 6);
+  want(s->d_bad, sizeof(unsigned int));
+  want(d.p1w, sizeof(double) * 128);
+  want(d.p1w_f, sizeof(float) * 128);
+  size_t total = 0;
+  for (const Part& t : parts) total += t.bytes;
+  void* slab = nullptr;
+  st = sim_alloc(s, &slab, total);
+  if (st != HEAT_OK) goto fail;
+  {
+    char* at = static_cast<char*>(slab);
+    for (const Part& t : parts) {
+      *t.field = at;
+      at += t.bytes;
+    }
+  }
   d.rc32[0] = d.r32;
   d.wc32[0] = d.q32;
   d.sc32[0] = d.d32[0];
   d.sc32[1] = d.d32[1];
-  s->iters_log_cap = 4096;
-  ALLOC(d.iters_log, sizeof(int) * s->iters_log_cap, int*);
-  d.iters_log_len = s->iters_log_cap;
-  ALLOC(s->d_dev, sizeof(SimDev), SimDev*);
-  ALLOC(s->d_sc, sizeof(SimScalars), SimScalars*);
-  ALLOC(s->d_q6, sizeof(double) * 6, double*);
-  ALLOC(s->d_bad, sizeof(unsigned int), unsigned int*);
-  ALLOC(d.p1w, sizeof(double) * 128, const double*);
-  ALLOC(d.p1w_f, sizeof(float) * 128, const float*);
-#undef ALLOC
   d.sc = s->d_sc;
   if (cudaMallocHost((void**)&s->h_sc, sizeof(SimScalars)) != cudaSuccess) {
     cudaGetLastError();
@@ -417,13 +432,12 @@ extern "C" heat_status heat_sim_create(const heat_mesh* mesh, const heat_bc* bc,
   reset_scalars(s->h_sc);
   {
     // default state: rho_c = k = 1, U^0 = 0 (Dirichlet nodes at their values)
-    std::vector<double2> ones((size_t)s->ne, make_double2(1.0, 1.0));
     double p1w[128];
     float p1w_f[128];
     p1_box_matrices(hx, hy, hz, p1w, p1w + 64);
     for (int t = 0; t < 128; ++t) p1w_f[t] = (float)p1w[t];
-    if (cudaMemcpy((void*)d.coef, ones.data(), (size_t)s->ne * sizeof(double2), cudaMemcpyHostToDevice) != cudaSuccess ||
-        cudaMemsetAsync(d.vec64[0], 0, N8, s->stream) != cudaSuccess ||
+    k_fill_ones<<<grid_for(s->ne, 256), 256, 0, s->stream>>>(const_cast<double2*>(d.coef), s->ne);
+    if (cudaGetLastError() != cudaSuccess || cudaMemsetAsync(d.vec64[0], 0, N8, s->stream) != cudaSuccess ||
         cudaMemsetAsync(d.vec64[1], 0, N8, s->stream) != cudaSuccess ||
         cudaMemsetAsync(d.vec64[2], 0, N8, s->stream) != cudaSuccess ||
         cudaMemsetAsync(d.d[0], 0, N8, s->stream) != cudaSuccess ||
@@ -558,23 +572,29 @@ extern "C" heat_status heat_set_state(heat_sim* s, const double* u, int on_devic
     for (long long n = 0; n < s->nn; ++n)
       if (!std::isfinite(u[n])) return set_error(HEAT_ERR_NONFINITE, "heat_set_state: non-finite value at node %lld", n);
   }
-  heat_status st = sim_read_scalars(s);
-  if (st != HEAT_OK) return st;
+  if (!on_device) {
+    heat_status st = copy_in(s, s->dev.vec64[0], u, (size_t)s->nn * 8, 0);
+    if (st != HEAT_OK) return st;
+    u = s->dev.vec64[0];
+  }
   reset_scalars(s->h_sc);
-  st = copy_in(s, s->dev.vec64[0], u, (size_t)s->nn * 8, on_device);
-  if (st != HEAT_OK) return st;
-  k_impose_dirichlet<<<grid_for(s->nn, 256), 256, 0, s->stream>>>(s->d_dev, s->dev.vec64[0]);
+  k_set_state<<<grid_for(s->nn, 256), 256, 0, s->stream>>>(s->d_dev, u, s->dev.vec64[0], *s->h_sc);
   CUDA_TRY(cudaGetLastError());
-  return sim_write_scalars(s);
+  CUDA_TRY(cudaStreamSynchronize(s->stream));  // the caller's array has been read
+  return HEAT_OK;
 }
 
 extern "C" heat_status heat_get_state(heat_sim* s, double* u, int on_device) {
   if (!s || !u) return set_error(HEAT_ERR_ARG, "heat_get_state: null argument");
+  if (on_device) {  // the slot of U^n is read on the device: one wait
+    k_get_state<<<grid_for(s->nn, 256), 256, 0, s->stream>>>(s->d_dev, u);
+    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(cudaStreamSynchronize(s->stream));
+    return HEAT_OK;
+  }
   heat_status st = sim_read_scalars(s);
   if (st != HEAT_OK) return st;
-  const double* src = s->dev.vec64[s->h_sc->iu1];
-  CUDA_TRY(cudaMemcpyAsync(u, src, (size_t)s->nn * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                           s->stream));
+  CUDA_TRY(cudaMemcpyAsync(u, s->dev.vec64[s->h_sc->iu1], (size_t)s->nn * 8, cudaMemcpyDeviceToHost, s->stream));
   CUDA_TRY(cudaStreamSynchronize(s->stream));
   return HEAT_OK;
 }

@@ -323,6 +323,36 @@ __global__ void __launch_bounds__(32 * kOpWarps, sizeof(T) == 8 ? 2 : 4)
       });
 }
 
+__global__ void k_fill_ones(double2* __restrict__ c, long long n) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    c[i] = make_double2(1.0, 1.0);
+}
+
+// U^0 into its slot (in place when u is the slot) with the Dirichlet values,
+// and the scalars of a simulation that has taken no step (the count of index
+// violations is kept).
+__global__ void k_set_state(const SimDev* __restrict__ sp, const double* u, double* u0, SimScalars fresh) {
+  const SimDev& s = *sp;
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < s.nn;
+       n += (long long)gridDim.x * blockDim.x) {
+    int i, j, k;
+    node_of(s, n, i, j, k);
+    if (is_dirichlet(s, i, j, k)) u0[n] = dirichlet_value(s, i, j, k);
+    else if (u != u0) u0[n] = u[n];
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    fresh.check_violations = s.sc->check_violations;
+    *s.sc = fresh;
+  }
+}
+__global__ void k_get_state(const SimDev* __restrict__ sp, double* __restrict__ out) {
+  const SimDev& s = *sp;
+  const double* __restrict__ u = s.vec64[s.sc->iu1];
+  for (long long n = blockIdx.x * (long long)blockDim.x + threadIdx.x; n < s.nn;
+       n += (long long)gridDim.x * blockDim.x)
+    out[n] = u[n];
+}
+
 // Overwrite Dirichlet nodes of u with their values.
 __global__ void k_impose_dirichlet(const SimDev* __restrict__ sp, double* __restrict__ u) {
   const SimDev& s = *sp;
