@@ -329,6 +329,16 @@ def fp64_peak_tflops(hg):
     return _FP64_PEAK
 
 
+def update_rate(prof: dict):
+    """GB/s of the update launch; None where the iteration has no update of its
+    own (held on the chip: ms_apply is then a whole iteration)."""
+    return prof["bytes_update"] / (prof["ms_update"] * 1e-3) / 1e9 if prof["ms_update"] > 0 else None
+
+
+def iteration_kernel(prof: dict, streaming: str) -> str:
+    return streaming if prof["ms_update"] > 0 else "k_cg_res (one iteration)"
+
+
 def fp64_roofline(hg, nodes: int, ms_apply: float) -> dict:
     """The FP64 apply against the measured FP64 FMA peak (its bound on this GPU)."""
     peak = fp64_peak_tflops(hg)
@@ -595,14 +605,14 @@ def run_batch(hg, torch, nsims: int, nsteps: int, stream, tune=True, fixed_tunin
                 "seconds": sec, "sims_per_s": nsims / sec, "dof_cg_iters_per_s": dof * its / sec,
                 "cg_iterations_per_sim_step": its / (nsims * nsteps),
                 "kernel_launches": stats[0]["kernel_launches"], "tuning": tuning,
-                "roofline": {"bound": "hbm", "kernel": "k_apply_dot<float>", "achieved": achieved, "peak": peak,
+                "roofline": {"bound": "hbm", "kernel": iteration_kernel(prof, "k_apply_dot<float>"), "achieved": achieved, "peak": peak,
                              "unit": "GB/s", "frac": achieved / peak,
                              "traffic": ncu_traffic("k_apply_dot<float>@lognormal_batch_256x40",
                                                    current_variant(hg, "fp32_refined")),
                              "ms_per_launch": prof["ms_apply"],
                              "algorithmic_bytes_per_launch": prof["bytes_apply"],
                              "update_kernel": {"ms_per_launch": prof["ms_update"],
-                                               "achieved": prof["bytes_update"] / (prof["ms_update"] * 1e-3) / 1e9}}}
+                                               "achieved": update_rate(prof)}}}
     finally:
         hg.heat_destroy_batch(b)
         for s in sims:
@@ -654,8 +664,7 @@ def run_layered(hg, torch, nsteps: int, stream, tune=True, cheb_degrees=(), cheb
                                                                            current_variant(hg, "fp32_refined"))
                                     if precision == "fp32_refined" else None},
                           "update": {"ms_per_launch": prof["ms_update"],
-                                     "achieved_gbs": prof["bytes_update"] / (prof["ms_update"] * 1e-3) / 1e9
-                                     if prof["ms_update"] > 0 else None}}
+                                     "achieved_gbs": update_rate(prof)}}
     u32, u64 = fields["fp32_refined"], fields["fp64"]
     out["final_field_rel_err_fp32_refined_vs_fp64"] = float(np.linalg.norm(u32 - u64) / np.linalg.norm(u64))
     if cheb_degrees:
@@ -1072,10 +1081,10 @@ def main():
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
                          "frac_of_nominal_7900_gbs": achieved / 7900.0,
-                         "kernel": kernel_key.split("@")[0], "peak_kind": f"{peak_kind} HBM copy (burst)",
+                         "kernel": iteration_kernel(prof, kernel_key.split("@")[0]), "peak_kind": f"{peak_kind} HBM copy (burst)",
                          "ms_per_launch": prof["ms_apply"], "algorithmic_bytes_per_launch": prof["bytes_apply"],
                          "update_kernel": {"ms_per_launch": prof["ms_update"], "algorithmic_bytes_per_launch": prof["bytes_update"],
-                                           "achieved": prof["bytes_update"] / (prof["ms_update"] * 1e-3) / 1e9}},
+                                           "achieved": update_rate(prof)}},
             "clocks": clocks,
             "fp64_path": fp64,
             "final_field_rel_err_vs_fp64_path": final_err,
