@@ -1612,11 +1612,12 @@ heat_status engine_autotune(heat_sim* const* sims, int nsims, int reps, int* bes
   std::vector<double> vbest(kNumVariants, 1e300);
   for (int v = -1; v < kNumVariants && st == HEAT_OK; ++v) {
     if (v >= 0 && prec == P_FP64 && !kVariants[v].f64[0]) continue;
-    // the on-chip solve does not depend on the segment size
+    // the on-chip solve does not depend on the segment size: it keeps the
+    // table's, which the FP64 apply and the streaming meshes also follow
     for (int si = 0; si < (v < 0 || kVariants[v].res ? 1 : 4) && st == HEAT_OK; ++si) {
       Tuning t = base;
       t.variant[prec] = v;
-      if (v >= 0) t.seg_nodes[bucket] = kSegs[si];
+      if (v >= 0 && !kVariants[v].res) t.seg_nodes[bucket] = kSegs[si];
       Engine* e = nullptr;
       st = engine_create(sims, nsims, prec, sims[0]->stream, &e, &t);
       if (st != HEAT_OK) break;
@@ -1648,7 +1649,7 @@ heat_status engine_autotune(heat_sim* const* sims, int nsims, int reps, int* bes
     }
   }
   for (int v : top) {
-    if (v < 0 || st != HEAT_OK) continue;
+    if (v < 0 || kVariants[v].res || st != HEAT_OK) continue;
     Tuning tv = base;
     tv.variant[prec] = v;
     for (int seg : wave_segments(sims, nsims, prec, tv, bucket)) {
