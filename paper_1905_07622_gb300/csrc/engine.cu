@@ -457,6 +457,7 @@ __global__ void k_count_unfinished(const SimDev* __restrict__ sims, int nsims, i
 struct Engine {
   std::vector<heat_sim*> sims;
   int prec = 0;
+  Tuning tuning{};  // the table the kernels come from, also when a preconditioner changes
   KernelSet ks{};
   cudaStream_t stream = nullptr;
   SimDev* d_sims = nullptr;
@@ -757,12 +758,12 @@ static heat_status engine_upload(Engine* e) {
     }
     e->h_sims.push_back(d);
   }
-  heat_status rst = res_schedule(e, has_res, has_stream, res_base);
-  if (rst != HEAT_OK) return rst;
   if ((long long)e->h_op.size() > e->cap_op || (long long)e->h_pw.size() > e->cap_pw ||
       (long long)e->h_aw.size() > e->cap_aw || (long long)e->h_ow.size() > e->cap_ow ||
       item_base > e->cap_partial)
     return set_error(HEAT_ERR_ARG, "engine: work lists exceed their capacity");
+  heat_status rst = res_schedule(e, has_res, has_stream, res_base);
+  if (rst != HEAT_OK) return rst;
   const int nwork[4] = {(int)e->h_op.size(), (int)e->h_pw.size(), (int)e->h_aw.size(), (int)e->h_ow.size()};
   CUDA_TRY(cudaMemcpyAsync(e->d_sims, e->h_sims.data(), sizeof(SimDev) * e->h_sims.size(), cudaMemcpyHostToDevice,
                            e->stream));
@@ -943,23 +944,46 @@ heat_status engine_create(heat_sim* const* sims, int nsims, int precision, cudaS
       return set_error(HEAT_ERR_ARG, "engine: the simulations of one batch must share the element type");
     }
   e->ncheb = members_ncheb(e);
-  e->ks = kernel_set(precision, tun ? *tun : tuning_get(), e->ncheb > 0, e->elem);
+  e->tuning = tun ? *tun : tuning_get();
+  e->ks = kernel_set(precision, e->tuning, e->ncheb > 0, e->elem);
   e->stream = stream;
-  // capacities: the geometry is a function of each mesh, so compute it
+  // Capacities: the geometry is a function of each mesh and of whether the
+  // member takes Chebyshev passes (they run on 16-lane segments where the plain
+  // apply may take 32-lane ones or the chip), and a member may change that at
+  // any time: each list holds the larger of the two forms.
   long long cap_op = 0, cap_pw = 0, cap_aw = 0, cap_ow = 0, cap_partial = 0, cap_tasks = 0;
   size_t cap_res = 0;
+  const KernelSet sets[2] = {kernel_set(precision, e->tuning, false, e->elem),
+                             kernel_set(precision, e->tuning, true, e->elem)};
+  const bool one_set = sets[0].apply_w == sets[1].apply_w && sets[0].dual == sets[1].dual && sets[0].res == sets[1].res;
+  struct Need {
+    int nx = 0, ny = 0, nz = 0;
+    long long op = 0, pw = 0, aw = 0, ow = 0, tasks = 0;
+    size_t res = 0;
+  } n;
   for (heat_sim* s : e->sims) {
-    SimDev d = s->dev;
-    tile_geometry(d, e->ks, e->prec == P_FP64);
-    cap_op += d.ntiles;
-    cap_pw += d.npw;
-    cap_aw += d.w_items;
-    cap_ow += d.o_items;
-    cap_partial += std::max(std::max(std::max(d.ntiles, d.npw), d.w_items), d.o_items);
-    d.cheb_m = 0;  // room for the on-chip solve also when the member starts with Chebyshev passes
-    d.res = res_plan(d, e->ks, precision == P_FP64);
-    cap_res += res_bytes(d, precision == P_FP64).total;
-    cap_tasks += d.res.g;
+    if (n.nx != s->dev.nx || n.ny != s->dev.ny || n.nz != s->dev.nz) {  // members of one size need the same
+      n = Need{s->dev.nx, s->dev.ny, s->dev.nz};
+      for (int k = 0; k < (one_set ? 1 : 2); ++k)
+        for (int cheb_m : {0, 2}) {
+          SimDev d = s->dev;
+          d.cheb_m = cheb_m;
+          tile_geometry(d, sets[k], precision == P_FP64);
+          n.op = std::max<long long>(n.op, d.ntiles);
+          n.pw = std::max<long long>(n.pw, d.npw);
+          n.aw = std::max<long long>(n.aw, d.w_items);
+          n.ow = std::max<long long>(n.ow, d.o_items);
+          n.res = std::max(n.res, res_bytes(d, precision == P_FP64).total);
+          n.tasks = std::max<long long>(n.tasks, d.res.g);
+        }
+    }
+    cap_op += n.op;
+    cap_pw += n.pw;
+    cap_aw += n.aw;
+    cap_ow += n.ow;
+    cap_partial += std::max(std::max(n.op, n.pw), std::max(n.aw, n.ow));
+    cap_res += n.res;
+    cap_tasks += n.tasks;
   }
   if (cap_op > (1LL << 30) || cap_pw > (1LL << 30) || cap_aw > (1LL << 30) || cap_ow > (1LL << 30)) {
     delete e;
@@ -1059,20 +1083,15 @@ heat_status engine_refresh(Engine* e) {
   const bool recapture = nch != e->ncheb;
   for (const heat_sim* s : e->sims)
     if (s->dev.elem != e->elem) return set_error(HEAT_ERR_ARG, "engine: a member changed its element type");
-  if ((nch > 0) != (e->ncheb > 0)) {
-    const KernelSet ks = kernel_set(e->prec, tuning_get(), nch > 0, e->elem);
-    bool same_shape = ks.wsx == e->ks.wsx && ks.wny == e->ks.wny && ks.wwarps == e->ks.wwarps &&
-                      ks.pw_chunk == e->ks.pw_chunk && (ks.apply_w != nullptr) == (e->ks.apply_w != nullptr);
-    for (int b = 0; b < 3; ++b) same_shape = same_shape && ks.seg_nodes[b] == e->ks.seg_nodes[b];
-    if (!same_shape)  // the work lists were sized for the old shape
-      return set_error(HEAT_ERR_ARG, "engine: the tuning table changed since the engine was built; rebuild it");
-    e->ks = ks;
-  }
+  if ((nch > 0) != (e->ncheb > 0)) e->ks = kernel_set(e->prec, e->tuning, nch > 0, e->elem);
   e->ncheb = nch;
   heat_status st = engine_upload(e);
-  if (st != HEAT_OK) return st;
-  st = loop_sync_reset(e);
-  if (st != HEAT_OK) return st;
+  if (st == HEAT_OK) st = loop_sync_reset(e);
+  if (st != HEAT_OK) {  // the graph is no longer that of the members: captured anew by the next refresh
+    if (e->gexec) cudaGraphExecDestroy(e->gexec);
+    e->gexec = nullptr;
+    return st;
+  }
   if (recapture || !e->gexec || e->grid_op != g_op || e->grid_pw != g_pw || e->grid_aw != g_aw || e->grid_ch != g_ch ||
       e->grid_ow != g_ow || e->has_res != h_res || e->has_stream != h_stream || e->grid_res != g_res ||
       e->smem_res != sm_res)

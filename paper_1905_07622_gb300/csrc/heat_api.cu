@@ -531,6 +531,18 @@ extern "C" heat_status heat_get_coeffs(heat_sim* s, double* rho_c, double* k, in
   return HEAT_OK;
 }
 
+// Brings the simulation's own engine in line with its descriptor. An engine
+// that cannot be is given up: the next step builds a new one.
+static heat_status refresh_own_engine(heat_sim* s) {
+  if (!s->eng) return HEAT_OK;
+  const heat_status st = engine_refresh(s->eng);
+  if (st != HEAT_OK) {
+    engine_destroy(s->eng);
+    s->eng = nullptr;
+  }
+  return st;
+}
+
 extern "C" heat_status heat_set_params(heat_sim* s, const heat_params* params) {
   if (!s) return set_error(HEAT_ERR_ARG, "heat_set_params: sim is NULL");
   heat_status st = check_params(params);
@@ -551,8 +563,7 @@ extern "C" heat_status heat_set_params(heat_sim* s, const heat_params* params) {
   }
   st = sim_refresh(s);
   if (st != HEAT_OK) return st;
-  if (s->eng) return engine_refresh(s->eng);
-  return HEAT_OK;
+  return refresh_own_engine(s);
 }
 
 extern "C" heat_status heat_cheb_interval(heat_sim* s, double* lam_lo, double* lam_hi) {
@@ -656,8 +667,7 @@ static heat_status ensure_log(heat_sim* s, int nsteps) {
   s->dev.iters_log_len = nsteps;
   st = sim_upload_desc(s);
   if (st != HEAT_OK) return st;
-  if (s->eng) return engine_refresh(s->eng);
-  return HEAT_OK;
+  return refresh_own_engine(s);
 }
 
 heat_status heat::sim_prepare_steps(heat_sim* s, int nsteps) {
