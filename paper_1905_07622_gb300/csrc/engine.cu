@@ -1320,16 +1320,22 @@ __global__ void k_flush_read(const uint4* __restrict__ p, size_t n, unsigned int
   if (acc == 0x9e3779b9u) *sink = acc;  // keeps the loads alive; practically never taken
 }
 
-// r[i] = a hash of i mapped to [-1, 1); *delta += sum r[i]^2 pinv[i].
+// r[i] = a hash of i mapped to [-1, 1), zero on Dirichlet rows as in a solve
+// (the on-chip forms count on it); *delta += sum r[i]^2 pinv[i].
 template <class T>
-__global__ void k_profile_seed(T* __restrict__ r, const T* __restrict__ pinv, long long n, double* delta) {
+__global__ void k_profile_seed(const SimDev* __restrict__ sp, T* __restrict__ r, const T* __restrict__ pinv,
+                               double* delta) {
+  const SimDev& s = *sp;
   double acc = 0.0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < s.nn;
+       i += (long long)gridDim.x * blockDim.x) {
+    int a, b, c;
+    node_of(s, i, a, b, c);
     unsigned int h = (unsigned int)i * 0x9E3779B1u;
     h ^= h >> 15;
     h *= 0x85EBCA77u;
     h ^= h >> 13;
-    const T v = (T)((double)(h >> 8) * (1.0 / 8388608.0) - 1.0);
+    const T v = is_dirichlet(s, a, b, c) ? T(0) : (T)((double)(h >> 8) * (1.0 / 8388608.0) - 1.0);
     r[i] = v;
     acc += (double)v * (double)v * (double)pinv[i];
   }
@@ -1352,12 +1358,12 @@ static heat_status profile_arm(Engine* e, double* d_delta, std::vector<double>& 
     heat_sim* s = e->sims[i];
     const int g = (int)std::min<long long>((s->nn + 255) / 256, 4LL * sm_count());
     if (e->prec == P_FP64) {
-      k_profile_seed<double><<<g, 256, 0, e->stream>>>(s->dev.r, s->dev.pinv, s->nn, d_delta + i);
+      k_profile_seed<double><<<g, 256, 0, e->stream>>>(s->d_dev, s->dev.r, s->dev.pinv, d_delta + i);
     } else {
       st = sim_read_scalars(s);
       if (st != HEAT_OK) return st;
       const int slot = e->ks.fused ? (s->h_sc->cgs & 1) : 0;
-      k_profile_seed<float><<<g, 256, 0, e->stream>>>(s->dev.rc32[slot], s->dev.pinv32, s->nn, d_delta + i);
+      k_profile_seed<float><<<g, 256, 0, e->stream>>>(s->d_dev, s->dev.rc32[slot], s->dev.pinv32, d_delta + i);
     }
   }
   if (cudaMemcpyAsync(h_delta.data(), d_delta, sizeof(double) * e->sims.size(), cudaMemcpyDeviceToHost,
