@@ -508,7 +508,8 @@ heat_status heat_profile_iteration(heat_sim* sim, int reps, void* flush, size_t 
                                    double* bytes_apply, double* bytes_update);
 /* The same for every member of a batch at once (each launch carries all of
  * them); needs a prior heat_batch_step and leaves the members' solver state
- * undefined. */
+ * undefined. In a batch of which some members are held on the chip and others
+ * stream, the streaming members' launches are timed and their bytes given. */
 heat_status heat_batch_profile_iteration(heat_batch* batch, int reps, void* flush, size_t flush_bytes,
                                          double* ms_apply, double* ms_update,
                                          double* bytes_apply, double* bytes_update);

@@ -1486,10 +1486,12 @@ heat_status engine_profile(Engine* e, int reps, void* flush, size_t flush_bytes,
   if (st != HEAT_OK) return st;
   *ms_apply = ta / reps;
   *ms_update = tu / reps;
-  // algorithmic bytes: every vector and coefficient touched once per launch
+  // algorithmic bytes: every vector and coefficient touched once per launch, of
+  // the members that the timed launches carry
   double ba = 0.0, bu = 0.0;
-  for (heat_sim* x : e->sims) {
-    const double n = (double)x->nn, ne = (double)x->ne;
+  for (size_t i = 0; i < e->sims.size(); ++i) {
+    if (!on_chip && e->h_sims[i].res.g > 0) continue;
+    const double n = (double)e->sims[i]->nn, ne = (double)e->sims[i]->ne;
     if (e->prec == P_FP64) {
       ba += n * (3 * 8 + 2 * 8) + ne * 16;    // r, P^-1, d_old in; d, q out; (rho_c, k)
       bu += n * (2 * 8 + 8 + 2 * 8 + 8 + 8);  // x in/out, d, r in/out, q, P^-1
@@ -1527,10 +1529,11 @@ heat_status engine_time_iterations(Engine* e, int reps, double* ms_per_iter) {
   // short of the point where a seeded residual has converged to rounding
   constexpr int kChunk = 40;
   const bool persistent = e->ks.loop || (e->has_res && !e->has_stream);
+  const bool limited = e->ks.loop || e->has_res;  // launches that run several iterations
   const int per_tick = persistent ? kChunk : e->iters_per_tick;
   const int chunk_ticks = persistent ? 1 : std::max(1, kChunk / e->iters_per_tick);
-  if (persistent) {
-    heat_status st = loop_sync_reset(e, kChunk);
+  if (limited) {  // beside streaming members, one on the chip takes a tick's iterations too
+    heat_status st = loop_sync_reset(e, per_tick);
     if (st != HEAT_OK) return st;
   }
   cudaEvent_t a, b;
@@ -1571,7 +1574,7 @@ heat_status engine_time_iterations(Engine* e, int reps, double* ms_per_iter) {
   cudaEventDestroy(a);
   cudaEventDestroy(b);
   cudaFree(d_delta);
-  if (persistent) {
+  if (limited) {
     const heat_status st2 = loop_sync_reset(e);
     if (st == HEAT_OK) st = st2;
   }
