@@ -575,9 +575,10 @@ typedef struct heat_tuning {
 int heat_tuning_num_variants(void);
 /* Shape of variant v: segment width in nodes along x (one lane per node),
  * node rows along y per lane, warps per block, whether an FP64 kernel exists,
- * how its loads travel (0 = plain loads one level ahead into registers,
- * S >= 2 = each thread's own cp.async copies S-1 levels ahead into an S-stage
- * ring in shared memory), and whether it is a fused iteration (FP32 paths
+ * how its loads travel (0 = plain loads one level ahead into registers; -1 =
+ * the same where a mesh streams, while one that fits is held on the chip; S >= 2
+ * = each thread's own cp.async copies S-1 levels ahead into an S-stage ring in
+ * shared memory), and whether it is a fused iteration (FP32 paths
  * only: one kernel per CG iteration in the Chronopoulos-Gear arrangement of
  * PCG, which forms both inner products of an iteration in one reduction,
  * instead of an apply kernel and an update kernel). Any output may be NULL.

@@ -170,8 +170,8 @@ bool variant_info(int v, int info[6]) {
   info[1] = kVariants[v].ny;
   info[2] = kVariants[v].warps;
   info[3] = kVariants[v].f64[0] != nullptr;
-  info[4] = kVariants[v].stages;
-  info[5] = kVariants[v].fused || kVariants[v].res;  // one kernel runs whole iterations
+  info[4] = kVariants[v].res ? -1 : kVariants[v].stages;
+  info[5] = kVariants[v].fused;
   return true;
 }
 

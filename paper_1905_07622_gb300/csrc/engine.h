@@ -86,8 +86,8 @@ struct Tuning {
 };
 int size_bucket(long long nn);
 int num_variants();
-// {segment width, rows per thread, warps per block, has an FP64 kernel, cp.async stages,
-//  fused iteration kernel}
+// {segment width, rows per thread, warps per block, has an FP64 kernel, cp.async stages
+//  (-1: held on the chip where the mesh fits), fused iteration kernel}
 bool variant_info(int v, int info[6]);
 Tuning tuning_get();
 heat_status tuning_set(const Tuning& t);
