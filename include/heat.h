@@ -564,7 +564,8 @@ heat_status heat_probe_grid_barrier(int blocks_per_sm, int reps, double* us_per_
  *     unfinished simulations with HEAT_ERR_TIMEOUT). Only for the FP32
  *     paths (loop[HEAT_FP64] must be 0) with a register-prefetch variant
  *     (stages 0, not fused) on trilinear boxes without Chebyshev passes;
- *     elsewhere the flag is ignored. Default {0, 0, 0}. */
+ *     under variant 0 it takes the place of the on-chip solve and runs the
+ *     items of variant 15. Elsewhere the flag is ignored. Default {0, 0, 0}. */
 typedef struct heat_tuning {
   int variant[3];
   int seg_nodes[3];

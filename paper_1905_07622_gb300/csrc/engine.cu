@@ -361,21 +361,28 @@ static int occupancy(TileFn fn, int threads, int smem) {
   return occ;
 }
 
+// The register-prefetch variant with a separate update of variant v's shape
+// (variant 0, which streams as one, where there is none).
+static int plain_of(int v) {
+  const WVariant& f = kVariants[v];
+  for (int a = 0; a < kNumVariants; ++a)
+    if (!kVariants[a].fused && !kVariants[a].res && kVariants[a].stages == 0 && kVariants[a].sx == f.sx &&
+        kVariants[a].ny == f.ny && kVariants[a].warps == f.warps)
+      return a;
+  return 0;
+}
+
 // The kernels of precision prec under tuning table t. With Chebyshev passes
 // (cheb) a fused variant is replaced by the register-prefetch variant of the
 // same segment shape: the fused iteration has no place for the passes.
 static KernelSet kernel_set(int prec, const Tuning& t, bool cheb = false, int elem = E_Q1) {
   const int ei = elem == E_P1 ? 1 : 0;
   int variant = t.variant[prec];
-  if (cheb && variant >= 0 && variant < kNumVariants && kVariants[variant].fused) {
-    const WVariant& f = kVariants[variant];
-    int alt = -1;
-    for (int v = 0; v < kNumVariants && alt < 0; ++v)
-      if (!kVariants[v].fused && kVariants[v].stages == 0 && kVariants[v].sx == f.sx && kVariants[v].ny == f.ny &&
-          kVariants[v].warps == f.warps)
-        alt = v;
-    variant = alt >= 0 ? alt : 0;
-  }
+  // the persistent iteration: FP32 paths, trilinear boxes, no Chebyshev passes;
+  // the on-chip form makes way for the plain one of its shape
+  const bool loop = t.loop[prec] && prec != P_FP64 && elem == E_Q1 && !cheb;
+  if (loop && variant >= 0 && variant < kNumVariants && kVariants[variant].res) variant = plain_of(variant);
+  if (cheb && variant >= 0 && variant < kNumVariants && kVariants[variant].fused) variant = plain_of(variant);
   KernelSet k;
   if (elem == E_P1)
     k = prec == P_FP64 ? make_set<P_FP64, 16, 16, E_P1>()
@@ -397,9 +404,7 @@ static KernelSet kernel_set(int prec, const Tuning& t, bool cheb = false, int el
       k.cheb_w = prec == P_FP64 ? v.cheb64[ei] : v.cheb32[ei];
       if (k.apply_w_smem > 0)
         cudaFuncSetAttribute(k.apply_w, cudaFuncAttributeMaxDynamicSharedMemorySize, k.apply_w_smem);
-      // the persistent iteration: FP32 paths, trilinear boxes, register
-      // prefetch, separate update, no Chebyshev passes
-      if (t.loop[prec] && prec != P_FP64 && elem == E_Q1 && !cheb && !v.fused && !v.res && v.stages == 0)
+      if (loop && !v.fused && v.stages == 0)  // register prefetch, separate update
         k.loop = loop_kernel(v.sx, v.ny, v.warps, t.pw_quads[prec]);
       if (v.res) {
         res_kernel_set(k, false, elem);
