@@ -61,10 +61,12 @@ typedef enum {
 
 typedef enum {
   HEAT_FP64 = 0,         /* operator, vectors and dots in FP64 */
-  HEAT_FP32_REFINED = 1, /* FP32 operator/vectors, FP64 dots; outer refinement
-                            on FP64 vectors, its residual operator in
-                            double-float (pairs of floats, ~48 bits) */
-  HEAT_FP32_PLAIN = 2    /* FP32 operator/vectors, FP64 dots, no refinement */
+  HEAT_FP32_REFINED = 1, /* FP32 operator/vectors; dots FP32 within a warp and
+                            FP64 from there on (double-float, pairs of floats
+                            of ~48 bits, where a mesh is held on the chip);
+                            outer refinement on FP64 vectors, its residual
+                            operator in double-float */
+  HEAT_FP32_PLAIN = 2    /* the same operator, vectors and dots, no refinement */
 } heat_precision;
 
 /* Solver parameters. heat_params_default() fills the defaults in brackets. */

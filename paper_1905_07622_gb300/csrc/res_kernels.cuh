@@ -181,7 +181,16 @@ template <> struct Exch<double> {
 
 // The sums' arithmetic: FP64 on the FP64 path; on the FP32 path the warps'
 // FP32 sums are added in double-float (48 bits; FP64 adds on this GPU take 64
-// cycles of a scheduler each, and these chains are on the critical path).
+// cycles of a scheduler each, and these chains are on the critical path: 960
+// cycles a sum within a block against 1,900, a time step on 100^3 3.3% and one on
+// 80^3 4.7% slower with them). FP32's range would be lost with its width, so
+// the partials are scaled by the power of two nearest 1 / delta as the solve
+// is taken up (exact; r.z and d.q stay within a few powers of ten of delta).
+// The FP32 parts are no longer than the streaming kernels': r.z has two
+// partials a warp, of at most 10 + 6 additions in a row over 576 nodes (k_update:
+// 16 + 5 over 512). Relative error of r.z over a million random nodes, root mean
+// square: 0.9e-9 in k_update's order, 0.8e-9 in this one, 1.3e-9 with one partial
+// a warp; the double-float additions after it were exact.
 __device__ __forceinline__ DF res_xor(const DF& v, int o) {
   return DF(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
 }
@@ -208,6 +217,8 @@ __device__ __forceinline__ bool res_finite(const DF& v) { return isfinite(v.hi);
 __device__ __forceinline__ bool res_finite(double v) { return isfinite(v); }
 __device__ __forceinline__ bool res_positive(const DF& v) { return v.hi > 0.f; }
 __device__ __forceinline__ bool res_positive(double v) { return v > 0.0; }
+// v as it is kept between launches (SimScalars, FP64): where a launch ends does not show
+__device__ __forceinline__ DF res_kept(const DF& v) { return DF(v.to_double()); }
 // v <= t: the double-float form decides in FP32 unless the two are close
 __device__ __forceinline__ bool res_below(const DF& v, double t, float tf) {
   if (tf > 1e-30f && (v.hi > 1.001f * tf || v.hi < 0.999f * tf)) return v.hi < tf;
@@ -287,11 +298,13 @@ __device__ __forceinline__ bool res_all_sum(const S& v, ulonglong2* mail, int g,
 // Block-wide state of the running task (S: DF or double).
 template <class T, class S>
 struct ResShared {
-  T wsum[kResThreads / 32];
-  S delta, dq;
+  T wsum[2 * kResThreads / 32];
+  S delta, dq;      // in units of unit
   T alpha, beta;
-  double thresh;
+  double thresh;    // in units of unit
   float thresh_f;
+  T scale;          // 1 / unit
+  double unit;      // a power of two: FP32 of delta's size, FP64 1
   int go;  // what the next phase does: kGo, or how the task ends
   int iter, iter_step;
   unsigned int tag0;
@@ -441,14 +454,14 @@ __device__ __forceinline__ bool res_halo_fetch(const ResBox& b, const int4* srow
   return true;
 }
 
-// Sum of the warps' partials over the block, in every lane of warp 0.
-template <class T, class S, int NW>
-__device__ __forceinline__ S res_block_sum(const T (&wsum)[kResThreads / 32]) {
+// Sum of the warps' NP partials over the block, in every lane of warp 0.
+template <class T, class S, int NP>
+__device__ __forceinline__ S res_block_sum(const T* wsum) {
   const int lane = (int)threadIdx.x & 31;
-  static_assert(NW == 8, "every group of 8 lanes sums the same 8 partials");
-  S v = res_from(wsum[lane & 7], S(0));
+  static_assert(NP == 8 || NP == 16, "every group of NP lanes sums the same partials");
+  S v = res_from(wsum[lane & (NP - 1)], S(0));
 #pragma unroll
-  for (int o = 4; o > 0; o >>= 1) v = v + res_xor(v, o);
+  for (int o = NP / 2; o > 0; o >>= 1) v = v + res_xor(v, o);
   return v;
 }
 
@@ -502,7 +515,7 @@ template <class T, class S>
 __device__ __forceinline__ void res_finish(const SimDev& s, const ResShared<T, S>& sh, int go, bool after_alpha,
                                            unsigned int tag) {
   SimScalars* sc = s.sc;
-  sc->dq = to_d(sh.dq);
+  sc->dq = to_d(sh.dq) * sh.unit;
   if (!after_alpha) {
     fail(sc, res_finite(sh.dq) ? ST_BREAKDOWN : ST_NONFINITE);
   } else {
@@ -510,7 +523,7 @@ __device__ __forceinline__ void res_finish(const SimDev& s, const ResShared<T, S
     sc->restart = 0;
     sc->iter = sh.iter;
     sc->iter_step = sh.iter_step;
-    sc->delta = to_d(sh.delta);
+    sc->delta = to_d(sh.delta) * sh.unit;
     if (go != kEndResid) sc->beta = (double)sh.beta;
     if (go == kEndFailed) fail(sc, res_finite(sh.delta) ? ST_NOT_CONVERGED : ST_NONFINITE);
     else if (go == kEndOuter) sc->phase = PH_OUTER;
@@ -539,8 +552,18 @@ __device__ __forceinline__ bool res_open_task(const SimDev* __restrict__ sims, i
   __syncthreads();
   if (c.phase != PH_ITER) return false;
   if (tid == 0) {
-    sh.delta = res_from(__ldcg(&s.sc->delta), S(0));
-    sh.thresh = sizeof(T) == 8 ? __ldcg(&s.sc->thresh) : __ldcg(&s.sc->thresh_in);
+    const double delta = __ldcg(&s.sc->delta);
+    double inv = 1.0;
+    if (sizeof(T) == 4) {  // within what its reciprocal has as a normal float
+      const int e = min(max(((__double2hiint(delta) >> 20) & 0x7ff) - 1023, -120), 120);
+      inv = __hiloint2double((1023 - e) << 20, 0);
+      sh.unit = __hiloint2double((1023 + e) << 20, 0);
+    } else {
+      sh.unit = 1.0;
+    }
+    sh.scale = (T)inv;
+    sh.delta = res_from(delta * inv, S(0));
+    sh.thresh = (sizeof(T) == 8 ? __ldcg(&s.sc->thresh) : __ldcg(&s.sc->thresh_in)) * inv;
     sh.thresh_f = (float)sh.thresh;
     sh.iter_step = __ldcg(&s.sc->iter_step);
     sh.iter = c.iter;
@@ -941,7 +964,7 @@ __device__ __noinline__ void res_setup(const SimDev& s, const Ctl& c, const ResT
       px[u * TH] = make_float4(xv[0], xv[1], xv[2], xv[3]);
       *reinterpret_cast<float4*>(sr + 4 * qd) = make_float4(rv[0], rv[1], rv[2], rv[3]);
       const bool pub = xq < b.nx && (rt.w || (b.xl && xq == 0) || (b.xr && xq + 4 >= b.nx));
-sat[qd] = res_group(rt.x + xq, pub ? rt.y + xq : -4);
+      sat[qd] = res_group(rt.x + xq, pub ? rt.y + xq : -4);
     }
   }
 }
@@ -1015,7 +1038,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
       float acc = acc2.x + acc2.y;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) sh.wsum[warp] = acc;
+      if (lane == 0) sh.wsum[warp] = acc * sh.scale;
       __syncthreads();
       if (warp == 0) {
         const DF v = res_block_sum<float, DF, NW>(sh.wsum);
@@ -1033,7 +1056,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
       }
       const float alpha = sh.alpha;
       const float2 ma = f2(-alpha, -alpha);
-      float2 z[MAXQ][2], racc = f2(0.f, 0.f);
+      float2 z[MAXQ][2], racc[2] = {f2(0.f, 0.f), f2(0.f, 0.f)};
 #pragma unroll
       for (int u = 0; u < MAXQ; ++u) {
         const int qd = tn + u * TH;
@@ -1055,8 +1078,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
           *reinterpret_cast<float4*>(sr + 4 * qd) = make_float4(r0.x, r0.y, r1.x, r1.y);
           z[u][0] = __fmul2_rn(r0, f2(pv[u].x, pv[u].y));
           z[u][1] = __fmul2_rn(r1, f2(pv[u].z, pv[u].w));
-          racc = __ffma2_rn(r0, z[u][0], racc);
-          racc = __ffma2_rn(r1, z[u][1], racc);
+          racc[u & 1] = __ffma2_rn(r0, z[u][0], racc[u & 1]);
+          racc[u & 1] = __ffma2_rn(r1, z[u][1], racc[u & 1]);
         }
       }
       if (tk.g > 1) {
@@ -1068,10 +1091,14 @@ __global__ void __launch_bounds__(kResThreads, 1)
           }
         }
       }
-      acc = racc.x + racc.y;
+      float2 rz = f2(racc[0].x + racc[0].y, racc[1].x + racc[1].y);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if (lane == 0) sh.wsum[warp] = acc;
+      for (int o = 16; o > 0; o >>= 1)
+        rz = __fadd2_rn(rz, f2(__shfl_xor_sync(0xffffffffu, rz.x, o), __shfl_xor_sync(0xffffffffu, rz.y, o)));
+      if (lane == 0) {
+        sh.wsum[warp] = rz.x * sh.scale;
+        sh.wsum[NW + warp] = rz.y * sh.scale;
+      }
       float4 xv[MAXQ];  // in flight during the sum
 #pragma unroll
       for (int u = 0; u < MAXQ; ++u)
@@ -1083,7 +1110,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
       for (int u = 0; u < HB; ++u) hat[u] = -1;
       bool ok = true;
       if (warp == 0) {
-        const DF v = res_block_sum<float, DF, NW>(sh.wsum);
+        const DF v = res_block_sum<float, DF, 2 * NW>(sh.wsum);
         DF tot = v;
         if (tk.g > 1) ok = res_all_sum<DF>(v, s.res_slots + res_mail(tk.g), tk.g, rank, tag, gs, tot);
         if (lane == 0) res_decide_beta<float, DF>(sh, s, ok, tot, false, round + 1 >= max_rounds);
@@ -1094,6 +1121,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
       go = sh.go;
       const float2 pa = f2(alpha, alpha);
       if (go == kGo) {
+        if (tid == 0) sh.delta = res_kept(sh.delta);  // its warp has no halo to write
         const float beta = sh.beta;
         const float2 be = f2(beta, beta);
         float4 dv[MAXQ];
