@@ -77,7 +77,11 @@ typedef struct {
   int max_iter;      /* CG iterations per step (all kinds), >= 1     [20000] */
   int resid_period;  /* true residual r = b - A x every this many
                         iterations (Algorithm 1 uses 50), >= 1       [50] */
-  int poll_period;   /* CG iterations queued between host polls      [32] */
+  int poll_period;   /* CG iterations queued between host polls      [32];
+                        at least the 6 of a tick. From the default on, meshes
+                        held on the chip are polled after three launches of a
+                        whole inner solve each, below it after one launch of
+                        poll_period iterations. Results do not depend on it */
   int precision;     /* heat_precision                               [HEAT_FP64] */
   double inner_rtol; /* FP32_REFINED: inner solve tolerance relative
                         to its own right-hand side                   [1e-5] */

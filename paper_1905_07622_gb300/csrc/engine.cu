@@ -533,6 +533,7 @@ static int tick_launches(const Engine* e) {
 // Rounds (CG iterations) one persistent launch runs at most: a solve's
 // inner iterations normally end it first, at a phase change.
 constexpr int kLoopRounds = 256;
+constexpr int kPollDefault = 32;  // poll_period's default; larger values poll as often
 constexpr int kResRounds = 4096;
 
 // Test hook (heat_debug_loop_wait): arrivals the barrier expects beyond the
@@ -1157,10 +1158,22 @@ __global__ void k_begin_steps(const SimDev* __restrict__ sims, int nsims, int ns
 }
 
 heat_status engine_step_all(Engine* e, int nsteps, heat_step_stats* stats, int reset_counters) {
-  int max_iter = 1, max_outer = 1, poll = 32;
+  int max_iter = 1, max_outer = 1, poll = kPollDefault;
   const bool waits = e->ks.loop || e->has_res;  // kernels whose bounded waits can give up
+  for (const heat_sim* s : e->sims) {
+    max_iter = std::max(max_iter, s->prm.max_iter);
+    max_outer = std::max(max_outer, s->prm.max_outer);
+    poll = std::min(poll, s->prm.poll_period);
+  }
+  // Iterations and ticks between two polls. Streaming: poll_period iterations.
+  // On the chip a launch carries a whole inner solve, and three ticks are a step
+  // of the refined path; below the default poll_period a launch ends after that
+  // many iterations and is polled after.
+  const bool chip = e->has_res && !e->has_stream;
+  const int rounds = !e->has_res || poll >= kPollDefault ? 0 : chip ? std::max(poll, e->iters_per_tick) : e->iters_per_tick;
+  const int ticks_per_poll = !chip ? std::max(1, poll / e->iters_per_tick) : poll >= kPollDefault ? 3 : 1;
   if (waits) {  // the bound and the test hook as they are now
-    heat_status st = loop_sync_reset(e);
+    heat_status st = loop_sync_reset(e, rounds);
     if (st != HEAT_OK) return st;
   }
   // the members' scalars are set on the device, all in one launch, after what
@@ -1172,14 +1185,6 @@ heat_status engine_step_all(Engine* e, int nsteps, heat_step_stats* stats, int r
   }
   k_begin_steps<<<1, 256, 0, e->stream>>>(e->d_sims, (int)e->sims.size(), nsteps, reset_counters);
   CUDA_TRY(cudaGetLastError());
-  for (const heat_sim* s : e->sims) {
-    max_iter = std::max(max_iter, s->prm.max_iter);
-    max_outer = std::max(max_outer, s->prm.max_outer);
-    poll = std::min(poll, s->prm.poll_period);
-  }
-  // the persistent form polls after as many graph launches as the tick form
-  // (on the chip a tick carries a whole inner solve: three ticks are a step)
-  const int ticks_per_poll = e->has_res && !e->has_stream ? 3 : std::max(1, poll / e->iters_per_tick);
   // Every tick advances each unfinished simulation by at least one CG
   // iteration or one phase change, so this bound is never reached by a
   // healthy solve; it turns a logic error into HEAT_ERR_TIMEOUT.

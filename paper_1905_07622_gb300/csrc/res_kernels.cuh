@@ -371,6 +371,13 @@ struct ResBox {
   }
 };
 
+// z = P^-1 r and d = z + beta d_old, each rounded once: the iteration's own
+// arithmetic, so a solve taken up by the next launch goes on bit for bit.
+__device__ __forceinline__ float res_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double res_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float res_fma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double res_fma(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // d on the box and its halo from the node vectors: P^-1 r + beta d_old
 // (restart: P^-1 r), zero outside the mesh. own node i of a row at d0 + i.
 template <class T>
@@ -390,7 +397,7 @@ __device__ __forceinline__ void res_load_d(const SimDev& s, const Ctl& c, const 
       const int i = t - d0;
       T v = T(0);
       if (in && i >= -1 && i <= b.nx && b.x0 + i >= 0 && b.x0 + i < b.X && HEAT_INDEX_OK(s.sc, m0 + i, s.nn))
-        v = pinv[m0 + i] * r[m0 + i] + beta * (rs ? T(0) : dold[m0 + i]);
+        v = res_fma(beta, rs ? T(0) : dold[m0 + i], res_mul(pinv[m0 + i], r[m0 + i]));
       sd[row * l.pd + t] = v;
     }
   }
@@ -1151,14 +1158,14 @@ __global__ void __launch_bounds__(kResThreads, 1)
           if (warp > 0) {
 #pragma unroll
             for (int u = 0; u < HB; ++u)
-              if (hat[u] >= 0) sd[hat[u]] = hz[u] + beta * sd[hat[u]];
+              if (hat[u] >= 0) sd[hat[u]] = res_fma(beta, sd[hat[u]], hz[u]);
           }
           // what the fetch has not covered
           for (int h = HB * (TH - 32) + tn; h < res_halo_cells(b) && ok; h += TH) {
             float z1[1];
             int a1[1];
             ok = res_halo_fetch<float, 1>(b, srow, shalo, h, 1 << 30, zx, tag, gs, z1, a1);
-            sd[a1[0]] = z1[0] + beta * sd[a1[0]];
+            sd[a1[0]] = res_fma(beta, sd[a1[0]], z1[0]);
           }
         }
         if (__syncthreads_or(!ok)) return;
@@ -1331,7 +1338,7 @@ __global__ void __launch_bounds__(kResThreads, 1)
         for (int u = 0; u < MAXN; ++u)
           if (tid + u * TH < nn) {
             r[u] -= alpha * q[u];
-            z[u] = p[u] * r[u];
+            z[u] = res_mul(p[u], r[u]);
             acc += r[u] * z[u];
             if (zo[u] >= 0) X::store(zx + 2 * (size_t)zo[u], z[u], tag);
           }
@@ -1362,18 +1369,18 @@ __global__ void __launch_bounds__(kResThreads, 1)
         const double beta = sh.beta;
 #pragma unroll
         for (int u = 0; u < MAXN; ++u)
-          if (tid + u * TH < nn) sd[at[u]] = z[u] + beta * sd[at[u]];
+          if (tid + u * TH < nn) sd[at[u]] = res_fma(beta, sd[at[u]], z[u]);
         if (rg.g > 1) {
           if (warp > 0) {
 #pragma unroll
             for (int u = 0; u < HB; ++u)
-              if (hat[u] >= 0) sd[hat[u]] = hz[u] + beta * sd[hat[u]];
+              if (hat[u] >= 0) sd[hat[u]] = res_fma(beta, sd[hat[u]], hz[u]);
           }
           for (int h = HB * (TH - 32) + tid; h < res_halo_cells(b) && ok; h += TH) {
             double z1[1];
             int a1[1];
             ok = res_halo_fetch<double, 1>(b, srow, shalo, h, 1 << 30, zx, tag, gs, z1, a1);
-            sd[a1[0]] = z1[0] + beta * sd[a1[0]];
+            sd[a1[0]] = res_fma(beta, sd[a1[0]], z1[0]);
           }
         }
         if (__syncthreads_or(!ok)) return;
