@@ -127,6 +127,9 @@ heat_status engine_step_all(Engine* e, int nsteps, heat_step_stats* stats, int r
 heat_status engine_launch_ticks(Engine* e, int nticks);
 // Phase of every simulation of the engine (host array of nsims ints); waits.
 heat_status engine_read_phases(Engine* e, int* phases);
+// Whether members are held on the chip: their ticks then carry up to an inner
+// solve each, not six iterations.
+bool engine_on_chip(const Engine* e);
 // Kernels launched so far by engine_launch_ticks / engine_step_all.
 long long engine_launches(const Engine* e);
 // Device bytes the engine needs for these simulations (work lists, partials).

@@ -103,10 +103,13 @@ static void finish_request(heat_server* srv, Req* q, heat_status status) {
   srv->cv_done.notify_all();
 }
 
-// Ticks launched between two reads of the members' phases (and admissions):
-// about 30 CG iterations at six per tick. Longer rounds keep a finished
-// request's slot idle for longer before the next admission takes it.
-constexpr int kTicksPerPoll = 5;
+// Ticks launched between two reads of the members' phases (and admissions).
+// Streaming: about 30 CG iterations at six per tick. With members on the chip a
+// tick is up to 48 iterations of them, mostly an inner solve, and three are a step
+// of the refined path (a burst of 8 mixed requests 35.2 ms, with five 36.7). Longer
+// rounds keep a finished request's slot idle for longer before the next
+// admission takes it.
+constexpr int kTicksPerPoll = 5, kChipTicksPerPoll = 3;
 // Work-list and descriptor capacity of a server engine relative to the member
 // set it is built for: later sets that fit run under the same captured graph.
 constexpr double kEngineHeadroom = 2.0;
@@ -227,7 +230,7 @@ static void worker_loop(heat_server* srv) {
       members_changed = false;
       if (srv->active.empty()) continue;
     }
-    heat_status s = engine_launch_ticks(eng, kTicksPerPoll);
+    heat_status s = engine_launch_ticks(eng, engine_on_chip(eng) ? kChipTicksPerPoll : kTicksPerPoll);
     phases.assign(srv->active.size(), 0);
     if (s == HEAT_OK) s = engine_read_phases(eng, phases.data());
     std::vector<Req*> keep;
