@@ -477,9 +477,14 @@ template <class T> struct IsThird<MarchQ1T<T, true>> : std::true_type {};
 // pre(node, in) loads what out needs at a node (in false: nothing to load, no
 // output); it runs before a level's arithmetic and out receives its result,
 // so those loads are in flight meanwhile.
-template <class T, int SX, int NY, class MC, class Src, class Pre, class Out>
+//
+// lev(t) runs after a level's outputs (t = 2, 3, ..; the same t in every lane).
+struct NoLev {
+  __device__ __forceinline__ void operator()(int) const {}
+};
+template <class T, int SX, int NY, class MC, class Src, class Pre, class Out, class Lev = NoLev>
 __device__ __forceinline__ void warp_tile_march_pre(const LaneGeo<NY>& lg, const MC& mc, Src& src, int tzl, Pre&& pre,
-                                                    Out&& out) {
+                                                    Out&& out, Lev&& lev = Lev{}) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NR = NY + 2;  // staged rows
   constexpr int NF = NY + 1;  // faces / element rows
@@ -567,6 +572,7 @@ __device__ __forceinline__ void warp_tile_march_pre(const LaneGeo<NY>& lg, const
             out(m, dir, nl + from_left, vprev[r - 1], got[r - 1]);
           }
         }
+        lev(t);
       }
     }
 #pragma unroll
@@ -579,10 +585,11 @@ __device__ __forceinline__ void warp_tile_march_pre(const LaneGeo<NY>& lg, const
 }
 
 struct NoPre {};
-template <class T, int SX, int NY, class MC, class Src, class Out>
-__device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC& mc, Src& src, int tzl, Out&& out) {
+template <class T, int SX, int NY, class MC, class Src, class Out, class Lev = NoLev>
+__device__ __forceinline__ void warp_tile_march(const LaneGeo<NY>& lg, const MC& mc, Src& src, int tzl, Out&& out,
+                                                Lev&& lev = Lev{}) {
   warp_tile_march_pre<T, SX, NY>(lg, mc, src, tzl, [](int, bool) { return NoPre{}; },
-                                 [&](int m, bool dir, T y, T v, NoPre) { out(m, dir, y, v); });
+                                 [&](int m, bool dir, T y, T v, NoPre) { out(m, dir, y, v); }, lev);
 }
 
 // The same contract on six-tetrahedra boxes (heat.h HEAT_ELEM_P1). Each lane
@@ -610,9 +617,9 @@ struct MarchP1 {
         kwy(sb * p1_consts<T>(s)[2]),
         kwz(sb * p1_consts<T>(s)[3]) {}
 };
-template <class T, int SX, int NY, class Src, class Out>
+template <class T, int SX, int NY, class Src, class Out, class Lev = NoLev>
 __device__ __forceinline__ void warp_tile_march_p1(const LaneGeo<NY>& lg, const MarchP1<T>& mc, Src& src, int tzl,
-                                                   Out&& out) {
+                                                   Out&& out, Lev&& lev = Lev{}) {
   constexpr unsigned FULL = 0xffffffffu;
   constexpr int NR = NY + 2;  // staged rows
   constexpr int NF = NY + 1;  // box rows
@@ -674,6 +681,7 @@ __device__ __forceinline__ void warp_tile_march_p1(const LaneGeo<NY>& lg, const 
           out(m, dir, y, prv[r]);
         }
       }
+      if (t >= 2) lev(t);
     }
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
@@ -686,30 +694,30 @@ __device__ __forceinline__ void warp_tile_march_p1(const LaneGeo<NY>& lg, const 
 // The march of element type E and its constants.
 template <int E, class T>
 using MarchE = typename std::conditional<E == E_P1, MarchP1<T>, MarchQ1<T>>::type;
-template <int E, class T, int SX, int NY, class Src, class Out>
+template <int E, class T, int SX, int NY, class Src, class Out, class Lev = NoLev>
 __device__ __forceinline__ void warp_march_c(const LaneGeo<NY>& lg, const MarchE<E, T>& mc, Src& src, int tzl,
-                                             Out&& out) {
+                                             Out&& out, Lev&& lev = Lev{}) {
   if constexpr (E == E_P1)
-    warp_tile_march_p1<T, SX, NY>(lg, mc, src, tzl, out);
+    warp_tile_march_p1<T, SX, NY>(lg, mc, src, tzl, out, lev);
   else
-    warp_tile_march<T, SX, NY>(lg, mc, src, tzl, out);
+    warp_tile_march<T, SX, NY>(lg, mc, src, tzl, out, lev);
 }
-template <int E, class T, int SX, int NY, class Src, class Out>
+template <int E, class T, int SX, int NY, class Src, class Out, class Lev = NoLev>
 __device__ __forceinline__ void warp_march_e(const LaneGeo<NY>& lg, const SimDev& s, Src& src, int tzl, T sa, T sb,
-                                             Out&& out) {
-  warp_march_c<E, T, SX, NY>(lg, MarchE<E, T>(s, sa, sb), src, tzl, out);
+                                             Out&& out, Lev&& lev = Lev{}) {
+  warp_march_c<E, T, SX, NY>(lg, MarchE<E, T>(s, sa, sb), src, tzl, out, lev);
 }
 
 // The register-prefetch form with functor loads (see RegSrc), for element E.
-template <int E, class T, int SX, int NY, class Coef, class Fetch, class Value, class Out>
+template <int E, class T, int SX, int NY, class Coef, class Fetch, class Value, class Out, class Lev = NoLev>
 __device__ __forceinline__ void warp_tile_op_e(const Geo& g, const SimDev& s, const Coef* __restrict__ coef,
                                                bool active, int i0, int j0, int k0, int tzl, T sa, T sb, bool mask,
-                                               Fetch&& fetch, Value&& value, Out&& out) {
+                                               Fetch&& fetch, Value&& value, Out&& out, Lev&& lev = Lev{}) {
   const LaneGeo<NY> lg(g, active, (int)threadIdx.x % SX, SX, i0, j0, mask, s.sc);
   using CoefT = typename std::remove_cv<typename std::remove_reference<decltype(coef[0])>::type>::type;
   RegSrc<T, NY, CoefT, typename std::remove_reference<Fetch>::type, typename std::remove_reference<Value>::type> src(
       coef, fetch, value, k0);
-  warp_march_e<E, T, SX, NY>(lg, s, src, tzl, sa, sb, out);
+  warp_march_e<E, T, SX, NY>(lg, s, src, tzl, sa, sb, out, lev);
 }
 
 }  // namespace heat
