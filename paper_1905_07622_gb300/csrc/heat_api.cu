@@ -351,10 +351,16 @@ extern "C" heat_status heat_sim_create(const heat_mesh* mesh, const heat_bc* bc,
     for (int t = 0; t < 4; ++t) d.p1c_f[t] = (float)d.p1c[t];
   }
   walsh_eigenvalues(hx, hy, hz, d.lam_m, d.lam_k);
-  d.sigma[0] = 12.0 / (hx * hx);
-  d.sigma[1] = 12.0 / (hy * hy);
-  d.sigma[2] = 12.0 / (hz * hz);
-  d.m43 = 4.0 / 3.0 * d.lam_m[0];
+  {
+    using L = long double;
+    const L m0 = (L)hx * hy * hz / 64, zeta = 12 / ((L)hz * hz);
+    const L sx = 12 / ((L)hx * hx), sy = 12 / ((L)hy * hy), sg[4] = {0, sx, sy, sx + sy};
+    d.m43 = (double)(4 * m0 / 3);
+    for (int q = 0; q < 4; ++q) {
+      d.tal[q] = (double)(m0 * (4 * sg[q] + zeta) / 3);
+      d.tbe[q] = (double)(m0 * (2 * sg[q] - zeta) / 3);
+    }
+  }
   for (int p = 0; p < 8; ++p) {
     d.mhat_f[p] = (float)d.mhat[p];
     d.khat_f[p] = (float)d.khat[p];

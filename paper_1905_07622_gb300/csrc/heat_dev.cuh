@@ -111,9 +111,9 @@ struct alignas(16) SimDev {  // 16-byte aligned: blocks copy it with uint4 loads
   // lam_k[w] = sum_d (w_d ? 2/h_d : 0) prod_{d' != d} (...) / 8.
   double lam_m[8], lam_k[8];
   float lam_m_f[8], lam_k_f[8];
-  // lam_w = lam_m[0] 3^-|w| (rho_c + k sum of sigma over w's differences) per
-  // unit scale: sigma[d] = 12 / h_d^2; m43 = 4/3 lam_m[0] (op_warp.cuh)
-  double sigma[3], m43;
+  // the march's form of them (op_warp.cuh), each rounded once: m43 = 4/3 m0,
+  // tal[q] = m0 (4 sigma_q + zeta) / 3, tbe[q] = m0 (2 sigma_q - zeta) / 3
+  double m43, tal[4], tbe[4];
   const double2* coef;        // (rho_c, k) per element
   const float2* coef32;
   double* vec64[4];           // U^{n-1}, U^{n-2}, x and spare (slots in SimScalars)

@@ -618,26 +618,19 @@ __device__ __forceinline__ void res_out(const ResTile& t, int r, float2 y, float
   if ((t.rows >> (r - 1)) & 1u) *reinterpret_cast<float2*>(q + (r - 1) * t.qrow) = y;
 }
 
-// Trilinear boxes. The Walsh eigenvalues of a box are
-//   lam_w = m0 3^-|w| (sa rho_c + sb k sigma_w), sigma_w = sum of 12 / h_d^2 over w's differences,
-// so with the factors 1/3 of x and y moved into the inverse butterflies (an
-// addition becomes a multiply-add, for free) an element's coefficients are
-//   A_q = R + K alpha_q, B_q = R / 2 + K beta_q,
-//   R = (4/3) m0 sa rho_c, K = m0 sb k, alpha_q = (4 sigma_q + zeta) / 3,
-//   beta_q = (2 sigma_q - zeta) / 3, zeta = 12 / h_z^2:
-// 4.5 packed operations per element instead of the 8 of march_coeffs. R and K
-// are formed once, when the block loads its coefficients.
+// Trilinear boxes, in the form of MarchQ1T<T, true> (op_warp.cuh): A_q = R + k al_q,
+// B_q = R / 2 + k be_q, 4.5 packed operations per element instead of the 8 of
+// march_coeffs. R is formed once, when the block loads its coefficients.
 struct ResQ1 {
   float al[4], be[4];
-  float ra, ka;  // R = ra rho_c, K = ka k
+  float ra, ka;  // the rho_c part is ra rho_c, the k part ka k
   __device__ __forceinline__ void set(const SimDev& s) {
-    const double sz = s.sigma[2], sg[4] = {0.0, s.sigma[0], s.sigma[1], s.sigma[0] + s.sigma[1]};
     for (int q = 0; q < 4; ++q) {
-      al[q] = (float)((4.0 * sg[q] + sz) / 3.0);
-      be[q] = (float)((2.0 * sg[q] - sz) / 3.0);
+      al[q] = (float)(s.tal[q] * s.theta);
+      be[q] = (float)(s.tbe[q] * s.theta);
     }
     ra = (float)(s.m43 * s.inv_dt);
-    ka = (float)(s.lam_m[0] * s.theta);
+    ka = 1.f;
   }
 };
 __device__ __forceinline__ float2 res_march(const ResTile& t, const ResQ1& mc, int tzl) {
