@@ -356,9 +356,12 @@ extern "C" heat_status heat_sim_create(const heat_mesh* mesh, const heat_bc* bc,
     const L m0 = (L)hx * hy * hz / 64, zeta = 12 / ((L)hz * hz);
     const L sx = 12 / ((L)hx * hx), sy = 12 / ((L)hy * hy), sg[4] = {0, sx, sy, sx + sy};
     d.m43 = (double)(4 * m0 / 3);
+    d.m43_f = (float)d.m43;
     for (int q = 0; q < 4; ++q) {
       d.tal[q] = (double)(m0 * (4 * sg[q] + zeta) / 3);
       d.tbe[q] = (double)(m0 * (2 * sg[q] - zeta) / 3);
+      d.tal_f[q] = (float)d.tal[q];
+      d.tbe_f[q] = (float)d.tbe[q];
     }
   }
   for (int p = 0; p < 8; ++p) {

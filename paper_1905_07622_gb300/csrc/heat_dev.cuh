@@ -114,6 +114,7 @@ struct alignas(16) SimDev {  // 16-byte aligned: blocks copy it with uint4 loads
   // the march's form of them (op_warp.cuh), each rounded once: m43 = 4/3 m0,
   // tal[q] = m0 (4 sigma_q + zeta) / 3, tbe[q] = m0 (2 sigma_q - zeta) / 3
   double m43, tal[4], tbe[4];
+  float m43_f, tal_f[4], tbe_f[4];
   const double2* coef;        // (rho_c, k) per element
   const float2* coef32;
   double* vec64[4];           // U^{n-1}, U^{n-2}, x and spare (slots in SimScalars)

@@ -437,11 +437,17 @@ struct MarchQ1T<T, true> {
   MarchQ1T() = default;
   __device__ __forceinline__ MarchQ1T(const SimDev& s, T sa, T sb) {
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      al[h] = V::make(sb * (T)s.tal[2 * h], sb * (T)s.tal[2 * h + 1]);
-      be[h] = V::make(sb * (T)s.tbe[2 * h], sb * (T)s.tbe[2 * h + 1]);
+    for (int h = 0; h < 2; ++h) {  // (a conversion is an FP64 instruction: floats have their own copies)
+      if constexpr (sizeof(T) == 8) {
+        al[h] = V::make(sb * s.tal[2 * h], sb * s.tal[2 * h + 1]);
+        be[h] = V::make(sb * s.tbe[2 * h], sb * s.tbe[2 * h + 1]);
+        ra = s.m43 * sa;
+      } else {
+        al[h] = V::make(sb * s.tal_f[2 * h], sb * s.tal_f[2 * h + 1]);
+        be[h] = V::make(sb * s.tbe_f[2 * h], sb * s.tbe_f[2 * h + 1]);
+        ra = s.m43_f * sa;
+      }
     }
-    ra = (T)s.m43 * sa;
   }
   template <class C>
   __device__ __forceinline__ void coeffs(const C& cf, T2 (&A)[2], T2 (&B)[2]) const {
