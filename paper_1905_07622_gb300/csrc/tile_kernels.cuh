@@ -199,11 +199,12 @@ __device__ __forceinline__ bool count_items(const SimDev& s, int n, int nitems, 
 }
 
 // A lane's sum over the outputs of a segment tile. FP32 sums up to 9 levels of 4
-// rows in a row; taller tiles fold them into a double-float every 8 levels and go
-// on in FP64 from the lane on, so that no FP32 sum is longer or spans more nodes
-// than those of the tiles of 9 levels. 200^3, 41 levels, relative error of d.q over
-// two million random nodes: 2.6e-9 with 164 terms in a row, 0.9e-9 with 36, 0.3e-9
-// folded, at 0.4% of a step (the fold is 7 operations of 4,000).
+// rows in a row; taller tiles fold them into a double-float every 8 levels, and
+// above 12 levels go on in FP64 from the lane on, so that no FP32 sum is longer or
+// spans many more nodes than those of the tiles of 9 levels. Relative error of d.q
+// over two million random nodes: 0.9e-9 with 36 terms in a row; 10 and 12 levels
+// folded 1.0e-9; 41 levels (200^3) 2.6e-9 with 164 terms in a row, 0.3e-9 folded,
+// at 0.4% of a step (the fold is 7 operations of 4,000).
 template <class T>
 struct LaneSum {
   T acc = T(0);
@@ -217,8 +218,8 @@ struct LaneSum {
 template <>
 struct LaneSum<float> {
   float acc = 0.f, hi = 0.f, lo = 0.f;
-  bool fold;
-  __device__ __forceinline__ explicit LaneSum(int levels) : fold(levels > 9) {}
+  bool fold, wide;
+  __device__ __forceinline__ explicit LaneSum(int levels) : fold(levels > 9), wide(levels > 12) {}
   __device__ __forceinline__ void level(int t) {  // after the outputs of level t - 1 (t from 2)
     if (fold && (t & 7) == 1) {
       const float sum = __fadd_rn(hi, acc), b = __fsub_rn(sum, hi);
@@ -228,11 +229,11 @@ struct LaneSum<float> {
     }
   }
   __device__ __forceinline__ void publish(const SimDev& s, int item, double* red) const {
-    if (fold) {
+    if (wide) {
       const double v[1] = {(df_widen(hi) + df_widen(lo)) + df_widen(acc)};
       publish_item<double, 1>(s, item, v, red);
     } else {
-      const float v[1] = {acc};
+      const float v[1] = {fold ? hi + (lo + acc) : acc};
       publish_item<float, 1>(s, item, v, red);
     }
   }
