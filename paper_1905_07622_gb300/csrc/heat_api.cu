@@ -1,7 +1,10 @@
 // C ABI of the solver (declared in include/heat.h): meshes, simulations,
 // the tick engine that drives the phase-gated kernels, and operator entry points.
+#include <cuda.h>
+
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
@@ -498,6 +501,29 @@ static heat_status copy_in(heat_sim* s, void* dst, const void* src, size_t bytes
   return HEAT_OK;
 }
 
+// Whether kernels may read or write `bytes` of doubles at a caller's device
+// address where they lie: on an 8-byte boundary and within one allocation. What
+// is not (or cannot be told) takes a copy, which any address suits and which
+// reports a range beyond its allocation instead of faulting on it.
+static bool in_place(const void* p, size_t bytes) {
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(double) != 0) return false;
+  using Range = CUresult (*)(CUdeviceptr*, size_t*, CUdeviceptr);
+  static const Range range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess) {
+      cudaGetLastError();
+      f = nullptr;
+    }
+    return reinterpret_cast<Range>(f);
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  const CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p);
+  return range && range(&base, &size, at) == CUDA_SUCCESS && at - base <= size && bytes <= size - (at - base);
+}
+
 extern "C" heat_status heat_set_coeffs(heat_sim* s, const double* rho_c, const double* k, int on_device) {
   if (!s || !rho_c || !k) return set_error(HEAT_ERR_ARG, "heat_set_coeffs: null argument");
   if (!on_device) {
@@ -508,17 +534,20 @@ extern "C" heat_status heat_set_coeffs(heat_sim* s, const double* rho_c, const d
         return set_error(HEAT_ERR_ARG, "heat_set_coeffs: coefficients must be > 0 (element %lld)", e);
     }
   }
-  // Device arrays are checked before anything live is changed; arrays of the
-  // host, checked above, are staged in the b and q work vectors (Ne < N). The
-  // setup kernel interleaves them into the live (rho_c, k) array.
-  if (!on_device) {
-    const size_t bytes = (size_t)s->ne * sizeof(double);
-    heat_status st = copy_in(s, s->dev.b, rho_c, bytes, 0);
+  // Device arrays are checked before anything live is changed, where they lie if
+  // kernels can read them there; others, and arrays of the host, checked above,
+  // are staged in the b and q work vectors (Ne < N). The setup kernel interleaves
+  // them into the live (rho_c, k) array.
+  const size_t bytes = (size_t)s->ne * sizeof(double);
+  if (!on_device || !in_place(rho_c, bytes) || !in_place(k, bytes)) {
+    heat_status st = copy_in(s, s->dev.b, rho_c, bytes, on_device);
     if (st != HEAT_OK) return st;
-    st = copy_in(s, s->dev.q, k, bytes, 0);
+    st = copy_in(s, s->dev.q, k, bytes, on_device);
     if (st != HEAT_OK) return st;
-    return sim_refresh(s, s->dev.b, s->dev.q);
+    rho_c = s->dev.b;
+    k = s->dev.q;
   }
+  if (!on_device) return sim_refresh(s, rho_c, k);
   CUDA_TRY(cudaMemsetAsync(s->d_bad, 0, sizeof(unsigned int), s->stream));
   k_check_coef_pair<<<grid_for(s->ne, 256), 256, 0, s->stream>>>(rho_c, k, s->ne, s->d_bad);
   CUDA_TRY(cudaGetLastError());
@@ -592,8 +621,8 @@ extern "C" heat_status heat_set_state(heat_sim* s, const double* u, int on_devic
     for (long long n = 0; n < s->nn; ++n)
       if (!std::isfinite(u[n])) return set_error(HEAT_ERR_NONFINITE, "heat_set_state: non-finite value at node %lld", n);
   }
-  if (!on_device) {
-    heat_status st = copy_in(s, s->dev.vec64[0], u, (size_t)s->nn * 8, 0);
+  if (!on_device || !in_place(u, (size_t)s->nn * 8)) {
+    heat_status st = copy_in(s, s->dev.vec64[0], u, (size_t)s->nn * 8, on_device);
     if (st != HEAT_OK) return st;
     u = s->dev.vec64[0];
   }
@@ -606,7 +635,7 @@ extern "C" heat_status heat_set_state(heat_sim* s, const double* u, int on_devic
 
 extern "C" heat_status heat_get_state(heat_sim* s, double* u, int on_device) {
   if (!s || !u) return set_error(HEAT_ERR_ARG, "heat_get_state: null argument");
-  if (on_device) {  // the slot of U^n is read on the device: one wait
+  if (on_device && in_place(u, (size_t)s->nn * 8)) {  // the slot of U^n is read on the device: one wait
     k_get_state<<<grid_for(s->nn, 256), 256, 0, s->stream>>>(s->d_dev, u);
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaStreamSynchronize(s->stream));
@@ -614,7 +643,8 @@ extern "C" heat_status heat_get_state(heat_sim* s, double* u, int on_device) {
   }
   heat_status st = sim_read_scalars(s);
   if (st != HEAT_OK) return st;
-  CUDA_TRY(cudaMemcpyAsync(u, s->dev.vec64[s->h_sc->iu1], (size_t)s->nn * 8, cudaMemcpyDeviceToHost, s->stream));
+  CUDA_TRY(cudaMemcpyAsync(u, s->dev.vec64[s->h_sc->iu1], (size_t)s->nn * 8,
+                           on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s->stream));
   CUDA_TRY(cudaStreamSynchronize(s->stream));
   return HEAT_OK;
 }
