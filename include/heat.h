@@ -287,10 +287,10 @@ void heat_destroy_server(heat_server* srv);
  * clears the hook. */
 heat_status heat_debug_fail_engine_builds(int n);
 /* Testing hook for the bounded waits of the persistent kernels (tuning loop,
- * and the on-chip solve of variants 0 and -1): engines built or refreshed
+ * and the on-chip solve of the default forms): engines built or refreshed
  * afterwards expect extra_arrivals (0 or 1) arrivals at each grid barrier or
- * all-sum beyond their blocks, so with 1 no wait ever completes, and bound one wait by limit_s seconds (0: the engine's own
- * bound of 1 s plus 50 ns per node). A wait that runs out ends the kernel;
+ * all-sum beyond their blocks, so with 1 no wait ever completes, and bound one
+ * wait by limit_s seconds (0: the engine's own bound of 1 s plus 50 ns per node). A wait that runs out ends the kernel;
  * the step then fails with HEAT_ERR_TIMEOUT and the GPU context stays
  * usable. HEAT_ERR_ARG unless extra_arrivals is 0 or 1 and
  * 0 <= limit_s <= 60. heat_debug_loop_wait(0, 0) restores the defaults. */
@@ -542,16 +542,21 @@ heat_status heat_probe_grid_barrier(int blocks_per_sm, int reps, double* us_per_
  * node count only, so a simulation gives bitwise the same results alone and in
  * any batch built under the same table.
  *   variant[p]: for heat_precision p, the warp-segment apply kernel variant
- *     (0 .. heat_tuning_num_variants()-1) or -1 for the block-tile apply.
- *     Default {-1, 0, 0}. Under variant 0 (FP32 paths) and -1 (FP64) a mesh
- *     that fits the GPU's shared memory (about 1.1 million nodes in FP32,
- *     130,000 in FP64) runs its whole inner solve in one persistent
- *     cooperative launch instead; larger meshes and Chebyshev members take
- *     the streaming kernels. Its waits are bounded like the grid barrier's
- *     (see loop): one that runs out fails the simulation with
- *     HEAT_ERR_TIMEOUT.
+ *     (0 .. heat_tuning_num_variants()-1) or -1. Default {-1, 0, 0}: the default
+ *     forms. Under them, 0 on the FP32 paths and -1 in FP64, a mesh that fits
+ *     the GPU's shared memory (cubes of up to 103 elements an edge, 1.1 million
+ *     nodes, in FP32; of 49, 0.12 million, in FP64) runs its whole inner solve in
+ *     one persistent cooperative launch; larger meshes and Chebyshev members
+ *     stream, FP32 in 16- or 32-lane segments of 4 rows by the mesh's width, FP64
+ *     in 16-lane ones. Variant 15 is variant 0 without the on-chip solve and
+ *     with 16-lane segments. -1 on the FP32 paths is the block-tile apply. The
+ *     on-chip solve's waits are bounded like the grid barrier's (see loop): one
+ *     that runs out fails the simulation with HEAT_ERR_TIMEOUT.
  *   seg_nodes[b]: output nodes per warp-segment tile for meshes of bucket b
- *     (N < 200000, N < 4000000, larger); 32 .. 2^20, default 512.
+ *     (N < 200000, N < 4000000, larger); 32 .. 2^20, default 512. Under the
+ *     default forms 512 leaves the tiles' height to an estimate of the launch's
+ *     time from the mesh and the GPU; any other size, and 512 under any other
+ *     variant, is taken as it is.
  *   pw_quads[p]: for heat_precision p, groups of 4 nodes each thread of the
  *     pointwise update kernel handles (1, 2 or 4; default {2, 4, 4}).
  *   open_w[p]: for heat_precision p, how the step-start and refinement
@@ -599,8 +604,8 @@ heat_status heat_tuning_set(const heat_tuning* t);
 /* Time CG iterations of this simulation as a solve runs them (the captured
  * tick graph of its engine, about `reps` iterations after 8 warm-up ones,
  * every iteration on a seeded residual that does not converge) for every
- * candidate (block tile; each variant with a segment size of 256, 512, 1024
- * or 2048 nodes; then, for the two fastest variants, the segment sizes whose work
+ * candidate (-1; the default form under the table's segment size; each other
+ * variant with a segment size of 256, 512, 1024 or 2048 nodes; then, for the two fastest variants, the segment sizes whose work
  * items fill whole waves of resident blocks best; then the pointwise item
  * sizes and the persistent iteration) on this simulation's mesh and
  * precision, and store the

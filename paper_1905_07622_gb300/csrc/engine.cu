@@ -29,7 +29,7 @@ struct KernelSet {
   TileFn open, apply, update;
   int sx, sy;
   int open_threads, apply_threads;
-  // warp-segment apply (FP32 paths); when set it replaces `apply`
+  // warp-segment apply; when set it replaces `apply` (always on the FP64 path)
   TileFn apply_w;
   int wsx, wny, wwarps;
   int pw_chunk;  // nodes per pointwise (k_update) work item
@@ -47,6 +47,7 @@ struct KernelSet {
   // the CG iterations of a tick as one persistent kernel (replaces the
   // apply and update launches when set; FP32 paths, register-prefetch apply)
   LoopFn loop = nullptr;
+  bool auto_seg = false;  // a default form: segment size kAutoSeg stands for the estimated best height
   bool dual = false;  // apply_w takes 16- and 32-lane segments, chosen per mesh (wsx for Chebyshev members)
   // the inner solve held on the chip: iterates the members whose mesh fits
   // (SimDev::res.g > 0); the others take apply and update
@@ -79,9 +80,14 @@ static TileFn open_w_kernel(int prec, int shape) {
 template <int P, int SX, int SY, int E = E_Q1>
 static KernelSet make_set() {
   using T = typename std::conditional<P == P_FP64, double, float>::type;
-  return {k_open<P, SX, SY, E>, k_apply_dot<T, SX, SY, E>, k_update<T, P, sizeof(T) == 4 ? 4 : 2>, SX, SY, SX * SY,
+  TileFn apply = nullptr, cheb = nullptr;  // FP64 has no block-tile form of these
+  if constexpr (P != P_FP64) {
+    apply = k_apply_dot<T, SX, SY, E>;
+    cheb = k_cheb<T, SX, SY, E>;
+  }
+  return {k_open<P, SX, SY, E>, apply, k_update<T, P, sizeof(T) == 4 ? 4 : 2>, SX, SY, SX * SY,
           SX * SY, nullptr, 0, 0, 0, pw_chunk(sizeof(T) == 4 ? 4 : 2), {512, 512, 512}, 0, false,
-          k_cheb<T, SX, SY, E>, nullptr};
+          cheb, nullptr};
 }
 
 // Warp-segment apply variants the tuner chooses from: segment width, rows per
@@ -155,10 +161,10 @@ static const WVariant kVariants[] = {
 constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
 
 // Process-wide tuning table, read when an engine is created: the warp apply
-// variant per precision (-1: the block-tile apply) and the segment tile size
+// variant per precision (-1: FP32 the block-tile apply, FP64 the default form) and the segment tile size
 // per mesh-size bucket. Both are fixed per simulation size, so results stay
 // bitwise identical alone and in batches built under the same table.
-constexpr int kAutoSeg = 512;  // the default segment size: levels per tile from pick_levels
+constexpr int kAutoSeg = 512;  // the default segment size: under the default variants, levels per tile from pick_levels
 static Tuning g_tuning = {{-1, 0, 0}, {kAutoSeg, kAutoSeg, kAutoSeg}, {2, 4, 4}, {2, 2, 2}, {0, 0, 0}};
 static std::mutex g_tuning_mu;
 
@@ -409,6 +415,7 @@ static KernelSet kernel_set(int prec, const Tuning& t, bool cheb = false, int el
       if (v.res) {
         res_kernel_set(k, false, elem);
         k.dual = true;
+        k.auto_seg = true;
       }
     }
   }
@@ -417,6 +424,7 @@ static KernelSet kernel_set(int prec, const Tuning& t, bool cheb = false, int el
     // of 4 rows (the FP64 pipe bounds the apply, and 4 rows compute 5 rows'
     // elements where 2 compute 3)
     res_kernel_set(k, true, elem);
+    k.auto_seg = true;
     // One block of 8 warps per SM: with two smaller ones, blocks that start
     // early (programmatic launch) pile up two to an SM while others stay empty
     // (100^3: 23.0 ms a step against 19.1 with the block tiles).
@@ -644,7 +652,8 @@ static void tile_geometry(SimDev& d, const KernelSet& ks, bool fp64) {
   d.w_ntx = d.w_nty = d.w_ntz = d.w_tz = d.w_ntiles = d.w_items = 0;
   if (ks.apply_w) {
     // segment tiles of about seg output nodes, at least 4 levels (2 extra levels
-    // per tile); the default size stands for the estimated best
+    // per tile); under the default variants the default size stands for the
+    // estimated best
     const int seg = ks.seg_nodes[size_bucket(d.nn)];
     // the narrower padded row; equal: whole lines
     const int pad16 = (d.nx + 1 + 13) / 14 * 14, pad32 = (d.nx + 1 + 29) / 30 * 30;
@@ -652,7 +661,7 @@ static void tile_geometry(SimDev& d, const KernelSet& ks, bool fp64) {
     d.w_ntx = (d.nx + 1 + d.w_sx - 3) / (d.w_sx - 2);
     d.w_nty = (d.ny + 1 + ks.wny - 1) / ks.wny;
     const int spc = ks.wwarps * (32 / d.w_sx);
-    const int tz0 = seg == kAutoSeg && ks.w_occ > 0
+    const int tz0 = ks.auto_seg && seg == kAutoSeg && ks.w_occ > 0
                         ? pick_levels((long long)d.w_ntx * d.w_nty, levels, spc, ks.w_occ, fp64 ? 1.0 : 0.34, 4.0, 96)
                         : std::max(4, std::min(levels, seg / ((d.w_sx - 2) * ks.wny)));
     d.w_ntz = (levels + tz0 - 1) / tz0;
@@ -749,7 +758,7 @@ static heat_status engine_upload(Engine* e) {
     d.partial = e->d_partial + 4 * item_base;
     item_base += std::max(std::max(std::max(d.ntiles, d.npw), d.w_items), d.o_items);
     const bool stream = d.res.g == 0;
-    // the block tiles also carry k_open's passes (k_apply_dot skips members on the chip)
+    // the block tiles also carry k_open's passes
     if (stream || !e->ks.open_w)
       for (int t = 0; t < d.ntiles; ++t) e->h_op.push_back(make_int2((int)i, t));
     if (stream) {
@@ -794,7 +803,7 @@ static heat_status engine_upload(Engine* e) {
   CUDA_TRY(cudaMemcpyAsync(e->d_nwork, nwork, sizeof(nwork), cudaMemcpyHostToDevice, e->stream));
   CUDA_TRY(cudaStreamSynchronize(e->stream));
   int occ_op = 1, occ_pw = 1, occ_aw = 1;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_op, e->ks.apply, e->ks.apply_threads, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_op, e->ks.apply ? e->ks.apply : e->ks.open, e->ks.apply_threads, 0);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_pw, e->ks.update, kPwThreads, 0);
   if (e->ks.apply_w)
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_aw, e->ks.apply_w, 32 * e->ks.wwarps, e->ks.apply_w_smem);

@@ -75,8 +75,9 @@ heat_status sim_setup_flux(heat_sim* s);
 // caller guarantees valid coefficients).
 heat_status sim_derive_async(heat_sim* s);
 
-// Kernel tuning: warp-apply variant per precision (-1: block-tile apply) and
-// segment tile size (nodes) per mesh-size bucket (size_bucket).
+// Kernel tuning: warp-apply variant per precision (-1: FP32 the block-tile
+// apply, FP64 the default form) and segment tile size (nodes) per mesh-size
+// bucket (size_bucket).
 struct Tuning {
   int variant[3];
   int seg_nodes[3];

@@ -3,8 +3,8 @@
 // coefficients in shared memory from the first iteration of an inner solve to
 // its last, instead of two launches per iteration that stream them through L2.
 //
-// What bounds an iteration of a mesh that fits (up to about 1.3 million
-// nodes: 152 SMs x 227 KB at about 24 bytes per node) is not bandwidth: the
+// What bounds an iteration of a mesh that fits (FP32: 152 SMs x 227 KB at about
+// 28 bytes per node with halos, cubes of up to 103 elements an edge) is not bandwidth: the
 // streaming kernels spend it on launch boundaries, on the descriptor and
 // scalar loads each block starts with, and on the last block's reduction tail
 // (fence, counter, partials, division: each an L2 round trip). Here the mesh
@@ -1199,8 +1199,8 @@ __global__ void __launch_bounds__(kResThreads, 1)
 // the whole cost: the factorised product takes about 60 operations per node
 // with its halo, a row of the assembled operator 27. Each block therefore
 // sums its nodes' 27 row coefficients over their elements once per launch,
-// keeps them in shared memory (216 bytes per node, so up to about 140,000
-// nodes fit) and applies them 27 FMAs per node and iteration. x, r, q, z and
+// keeps them in shared memory (216 bytes per node, so cubes of up to 49
+// elements an edge fit) and applies them 27 FMAs per node and iteration. x, r, q, z and
 // P^-1 stay in registers. Row layout: coefficient o = (ox+1) + 3 (oy+1) +
 // 9 (oz+1) of node n at sw[o * nodes + n].
 template <int E>

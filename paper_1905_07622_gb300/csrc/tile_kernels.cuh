@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(SX* SY) k_apply_dot(const SimDev* __restrict__
     cache_sim(sims, wi.x, cache, cur, dep);
     const SimDev& s = cache.s;
     const Ctl& c = cache.c;
-    if (c.phase != PH_ITER || s.res.g > 0) continue;  // res: iterated on the chip (k_cg_res)
+    if (c.phase != PH_ITER) continue;
     const Geo g(s);
     const TileCoords tc = tile_coords<SX, SY>(s, wi.y);
     // d = P^-1 r + beta d_old; after Chebyshev passes r is their P z, so d = z + beta d_old
