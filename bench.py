@@ -40,10 +40,12 @@ METRIC = "DOF*CG-iters/s"
 # of FP32 values with error-free sums and products (about 48 significant bits).
 DTYPE_DETAIL = {
     "fp64": "FP64 vectors, operator and dot products",
-    "fp32_refined": ("inner CG in FP32 (vectors and operator; dot products summed in FP32 per warp, then FP64); "
+    "fp32_refined": ("inner CG in FP32 (vectors and operator; dot products summed in FP32 per warp, then in FP64, or in "
+                     "double-float where the mesh is held on the chip); "
                      "outer refinement: FP64 solution, right-hand side and residual vectors with FP64 dot "
                      "products, the residual's operator b - A x evaluated in double-float (df64, ~48 bits)"),
-    "fp32_plain": "FP32 vectors and operator; dot products summed in FP32 per warp, then FP64",
+    "fp32_plain": ("FP32 vectors and operator; dot products summed in FP32 per warp, then in FP64, or in double-float "
+                   "where the mesh is held on the chip"),
 }
 UNIT = "DOF*iter/s"
 WORKLOAD = "inclusions_cube_100: Q1 100^3 (1,030,301 DOF), 200 spherical inclusions k=10 rho_c=3, flux pulse z=1 for 50 steps, dt=1e-3, theta=0.5, 300 steps per forward solve, rtol 1e-10"
@@ -318,6 +320,8 @@ def cheb_degrees(args):
 # (A, B, G, Tn), inverse y 4, node sums 5 = 67; the direction update
 # d = P^-1 r + beta d_old 3 and the dot product d.q 2. An FMA counts 2.
 FP64_APPLY_FLOPS_PER_NODE = 72
+# A whole iteration: the apply's and x += alpha d, r -= alpha q, z = P^-1 r, r.z.
+ITERATION_FLOPS_PER_NODE = FP64_APPLY_FLOPS_PER_NODE + 7
 _FP64_PEAK = None
 
 
@@ -337,11 +341,40 @@ def update_rate(prof: dict):
 
 def iteration_kernel(hg, prof: dict, precision: str, streaming: str) -> str:
     """The kernel `prof` timed: without an update of its own an iteration is one
-    launch of the fused form or a share of the on-chip solve (variant 0)."""
+    launch of the fused form or a share of the on-chip solve."""
     if prof["ms_update"] > 0:
         return streaming
-    v = hg.heat_tuning_get()["variant"][hg.PRECISIONS[precision]]
-    return "k_cg_res (one iteration)" if v <= 0 else "k_cg_iter"
+    if prof["bytes_apply"] > 0:
+        return "k_cg_iter"
+    return "k_cg_res64 (one iteration)" if precision == "fp64" else "k_cg_res (one iteration)"
+
+
+def apply_rate(prof: dict):
+    """GB/s of the apply (or fused) launch; None where the iteration is held on
+    the chip and moves no DRAM bytes of its own."""
+    return prof["bytes_apply"] / (prof["ms_apply"] * 1e-3) / 1e9 if prof["bytes_apply"] > 0 else None
+
+
+def fraction(rate, peak):
+    return rate / peak if rate is not None else None
+
+
+def iteration_roofline(hg, prof: dict, kernel: str, nodes: int, peak_gbs: float, peak_kind: str) -> dict:
+    """What bounds the iteration's main launch: HBM for the streaming kernels; on
+    the chip the FP32 pipe and the exchanges between blocks, so its arithmetic
+    against the measured FP32 FMA rate."""
+    out = {"kernel": kernel, "ms_per_launch": prof["ms_apply"]}
+    rate = apply_rate(prof)
+    if rate is None:
+        peak = hg.heat_probe_fma_rate(False, 5)
+        tflops = ITERATION_FLOPS_PER_NODE * nodes / (prof["ms_apply"] * 1e-3) / 1e12
+        return dict(out, bound="fp32 issue and exchange latency", achieved=tflops, peak=peak, unit="TFLOP/s",
+                    frac=tflops / peak, flops_per_node=ITERATION_FLOPS_PER_NODE, traffic=None,
+                    peak_kind="measured FP32 FMA rate (heat_probe_fma_rate, this run)")
+    return dict(out, bound="hbm", achieved=rate, peak=peak_gbs, unit="GB/s", frac=rate / peak_gbs,
+                peak_kind=f"{peak_kind} HBM copy (burst)", algorithmic_bytes_per_launch=prof["bytes_apply"],
+                update_kernel={"ms_per_launch": prof["ms_update"], "algorithmic_bytes_per_launch": prof["bytes_update"],
+                               "achieved": update_rate(prof)})
 
 
 def fp64_roofline(hg, nodes: int, ms_apply: float) -> dict:
@@ -604,20 +637,16 @@ def run_batch(hg, torch, nsims: int, nsteps: int, stream, tune=True, fixed_tunin
         torch.cuda.nvtx.range_push("roofline_batch")  # ncu captures filter on this range
         prof = hg.heat_batch_profile_iteration(b, 20, flush)
         torch.cuda.nvtx.range_pop()
-        peak, _ = measured_peaks()
-        achieved = prof["bytes_apply"] / (prof["ms_apply"] * 1e-3) / 1e9
+        peak, peak_kind = measured_peaks()
+        rated = iteration_roofline(hg, prof, iteration_kernel(hg, prof, "fp32_refined", "k_apply_dot<float>"),
+                                   nsims * dof, peak, peak_kind)
+        if rated["bound"] == "hbm":
+            rated["traffic"] = ncu_traffic("k_apply_dot<float>@lognormal_batch_256x40", current_variant(hg, "fp32_refined"))
         return {"workload": f"{nsims} x lognormal_cube_40 (68,921 DOF each), {nsteps} steps, dt=2e-3, theta=0.5, rtol 1e-10, fp32_refined",
                 "seconds": sec, "sims_per_s": nsims / sec, "dof_cg_iters_per_s": dof * its / sec,
                 "cg_iterations_per_sim_step": its / (nsims * nsteps),
                 "kernel_launches": stats[0]["kernel_launches"], "tuning": tuning,
-                "roofline": {"bound": "hbm", "kernel": iteration_kernel(hg, prof, "fp32_refined", "k_apply_dot<float>"), "achieved": achieved, "peak": peak,
-                             "unit": "GB/s", "frac": achieved / peak,
-                             "traffic": ncu_traffic("k_apply_dot<float>@lognormal_batch_256x40",
-                                                   current_variant(hg, "fp32_refined")),
-                             "ms_per_launch": prof["ms_apply"],
-                             "algorithmic_bytes_per_launch": prof["bytes_apply"],
-                             "update_kernel": {"ms_per_launch": prof["ms_update"],
-                                               "achieved": update_rate(prof)}}}
+                "roofline": rated}
     finally:
         hg.heat_destroy_batch(b)
         for s in sims:
@@ -658,13 +687,14 @@ def run_layered(hg, torch, nsteps: int, stream, tune=True, cheb_degrees=(), cheb
             torch.cuda.nvtx.range_push(f"roofline_layered_{precision}")  # ncu captures filter on this range
             prof = hg.heat_profile_iteration(s.sim, 20, flush)
             torch.cuda.nvtx.range_pop()
-        achieved = prof["bytes_apply"] / (prof["ms_apply"] * 1e-3) / 1e9
+        achieved = apply_rate(prof)
         if precision == "fp64":
             out["fp64_roofline"] = fp64_roofline(hg, p.n_nodes, prof["ms_apply"])
         out[precision] = {"seconds": sec, "ms_per_step": sec * 1e3 / nsteps, "cg_iterations": st["iters"],
                           "dof_cg_iters_per_s": p.n_nodes * st["iters"] / sec, "kernel_tuning": tuning,
                           "apply": {"ms_per_launch": prof["ms_apply"], "achieved_gbs": achieved, "peak_gbs": peak,
-                                    "frac": achieved / peak, "algorithmic_bytes_per_launch": prof["bytes_apply"],
+                                    "frac": fraction(achieved, peak),
+                                    "algorithmic_bytes_per_launch": prof["bytes_apply"],
                                     "traffic": ncu_traffic("k_apply_dot<float>@layered_cube_200",
                                                                            current_variant(hg, "fp32_refined"))
                                     if precision == "fp32_refined" else None},
@@ -756,11 +786,11 @@ def run_p1(hg, torch, nsteps: int, stream, table=None):
             torch.cuda.nvtx.range_push(f"roofline_{element}")
             prof = hg.heat_profile_iteration(s.sim, 40, flush)
             torch.cuda.nvtx.range_pop()
-        achieved = prof["bytes_apply"] / (prof["ms_apply"] * 1e-3) / 1e9
+        achieved = apply_rate(prof)
         out[element] = {"ms_per_step": sec * 1e3 / nsteps, "cg_iterations": st["iters"], "status": st["status"],
                         "dof_cg_iters_per_s": p.n_nodes * st["iters"] / sec,
                         "apply": {"ms_per_launch": prof["ms_apply"], "achieved_gbs": achieved, "peak_gbs": peak,
-                                  "frac": achieved / peak, "algorithmic_bytes_per_launch": prof["bytes_apply"]},
+                                  "frac": fraction(achieved, peak), "algorithmic_bytes_per_launch": prof["bytes_apply"]},
                         "update_ms_per_launch": prof["ms_update"]}
     return out
 
@@ -1041,9 +1071,11 @@ def main():
     prof_kernel = iteration_kernel(hg, prof, args.precision, f"k_apply_dot<{'double' if args.precision == 'fp64' else 'float'}>")
     torch.cuda.nvtx.range_pop()
     peak, peak_kind = measured_peaks()
-    achieved = prof["bytes_apply"] / (prof["ms_apply"] * 1e-3) / 1e9
-    kernel_key = f"k_apply_dot<{'double' if args.precision == 'fp64' else 'float'}>@inclusions_cube_100"
-    traffic = ncu_traffic(kernel_key, current_variant(hg, args.precision))
+    rated = iteration_roofline(hg, prof, prof_kernel, nn, peak, peak_kind)
+    if rated["bound"] == "hbm":
+        kernel_key = f"k_apply_dot<{'double' if args.precision == 'fp64' else 'float'}>@inclusions_cube_100"
+        rated["traffic"] = ncu_traffic(kernel_key, current_variant(hg, args.precision))
+        rated["frac_of_nominal_7900_gbs"] = rated["achieved"] / 7900.0
 
     batched = serving = layered = mh = p1 = None
     if rank == 0 and args.batch_sims > 0:
@@ -1084,13 +1116,7 @@ def main():
             "e2e": {"value": value_e2e, "unit": UNIT,
                     "h2d_bytes_per_step": 8 * (2 * ne + nn), "d2h_bytes_per_step": 8 * nn},
             "gpu_launches": launches,
-            "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak, "traffic": traffic,
-                         "frac_of_nominal_7900_gbs": achieved / 7900.0,
-                         "kernel": prof_kernel, "peak_kind": f"{peak_kind} HBM copy (burst)",
-                         "ms_per_launch": prof["ms_apply"], "algorithmic_bytes_per_launch": prof["bytes_apply"],
-                         "update_kernel": {"ms_per_launch": prof["ms_update"], "algorithmic_bytes_per_launch": prof["bytes_update"],
-                                           "achieved": update_rate(prof)}},
+            "roofline": rated,
             "clocks": clocks,
             "fp64_path": fp64,
             "final_field_rel_err_vs_fp64_path": final_err,

@@ -507,7 +507,9 @@ heat_status heat_apply_dot_noalloc(int nx, int ny, int nz, const double extent[3
  * launch. If flush != NULL, flush_bytes of it are overwritten before every
  * timed launch (to evict L2). Outputs the mean ms per launch of each kernel
  * and their algorithmic DRAM bytes per launch (vectors and coefficients each
- * touched once). Needs a prior heat_step on the sim; leaves its solver state
+ * touched once). Of a mesh held on the chip ms_apply is a whole iteration (a
+ * launch of 40 over 40), and the others are 0: the iteration has no DRAM
+ * traffic of its own. Needs a prior heat_step on the sim; leaves its solver state
  * undefined (call heat_set_state before stepping again). */
 heat_status heat_profile_iteration(heat_sim* sim, int reps, void* flush, size_t flush_bytes,
                                    double* ms_apply, double* ms_update,

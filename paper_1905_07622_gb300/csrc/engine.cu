@@ -1529,7 +1529,8 @@ heat_status engine_profile(Engine* e, int reps, void* flush, size_t flush_bytes,
       bu += n * (2 * 4 + 4 + 2 * 4 + 4 + 4);
     }
   }
-  *bytes_apply = on_chip ? ba + bu : ba;
+  // an iteration on the chip has no DRAM traffic of its own
+  *bytes_apply = on_chip ? 0.0 : ba;
   *bytes_update = on_chip ? 0.0 : bu;
   return HEAT_OK;
 }
