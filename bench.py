@@ -530,13 +530,27 @@ def autotune(hg, p, precision, stream, reps=40):
     return {"table": table, "best_ms_per_cg_iteration": ms}
 
 
+def plain_variant(hg, v: int) -> int:
+    """The register-prefetch variant with an update of its own of v's shape (v where none is)."""
+    if v < 0:
+        return v
+    info = [hg.heat_tuning_variant(k) for k in range(hg.heat_tuning_num_variants())]
+    shape = ("seg_width", "rows", "warps")
+    for k, i in enumerate(info):
+        if i["stages"] == 0 and not i["fused"] and all(i[a] == info[v][a] for a in shape):
+            return k
+    return v
+
+
 def run_persistent(hg, torch, stream, headline_table, batch_table, nsteps_single=30, nsims=256, nsteps_batch=10):
     """The persistent inner iteration (tuning loop = 1: one cooperative kernel
     per tick that runs the iterations with a grid barrier after each phase)
     against the replayed tick graph (an apply and an update launch per
     iteration), each under its own table, on the first steps of the headline
-    workload and of the batched one. Same work items, so with equal item sizes
-    the fields are bitwise equal (checked here on the headline)."""
+    workload and of the batched one. A variant without a persistent form (the
+    on-chip solve, the fused and the staged ones) gives way to the plain one of
+    its shape on both sides. Same work items, so with equal item sizes the
+    fields are bitwise equal (checked here on the headline)."""
     import numpy as np
     import workloads as W
     base = hg.heat_tuning_get()
@@ -545,6 +559,7 @@ def run_persistent(hg, torch, stream, headline_table, batch_table, nsteps_single
     def table(t, loop, quads=None):
         t = {k: list(v) for k, v in t.items()}
         t["loop"][pid] = loop
+        t["variant"][pid] = plain_variant(hg, t["variant"][pid])
         if quads is not None:
             t["pw_quads"][pid] = quads
         return t
