@@ -285,8 +285,8 @@ __global__ void k_reciprocal(const double* __restrict__ a, double* __restrict__ 
 //   OP_A: y = A' x, the eliminated operator padded with the identity
 //   OP_GENERAL: y = (sa M + sb K) x, no elimination
 //   OP_RHS: b = L u + F^n - z on free rows, g on Dirichlet rows
-// Measured (one GB300, gathered -> marched): FP32 A' x on 200^3 778 -> 55 us
-// (130 MB, 2.4 TB/s), FP64 right-hand side on 100^3 385 -> 172 us (bound by the
+// Measured (one GB300, gathered -> marched): FP32 A' x on 200^3 778 -> 54 us
+// (130 MB, 2.4 TB/s), FP64 right-hand side on 100^3 385 -> 166 us (bound by the
 // FP64 pipe), FP64 A' x on 33x21x17 18.4 -> 12.3 us (one wave of short tiles).
 enum OpMode : int { OP_A = 0, OP_GENERAL = 1, OP_RHS = 2 };
 struct OpTiles {
