@@ -290,10 +290,11 @@ heat_status heat_debug_fail_engine_builds(int n);
  * and the on-chip solve of the default forms): engines built or refreshed
  * afterwards expect extra_arrivals (0 or 1) arrivals at each grid barrier or
  * all-sum beyond their blocks, so with 1 no wait ever completes, and bound one
- * wait by limit_s seconds (0: the engine's own bound of 1 s plus 50 ns per node). A wait that runs out ends the kernel;
- * the step then fails with HEAT_ERR_TIMEOUT and the GPU context stays
- * usable. HEAT_ERR_ARG unless extra_arrivals is 0 or 1 and
- * 0 <= limit_s <= 60. heat_debug_loop_wait(0, 0) restores the defaults. */
+ * wait by limit_s seconds (0: the engine's own bound of 1 s plus 50 ns per
+ * node). A wait that runs out ends the kernel; the step then fails with
+ * HEAT_ERR_TIMEOUT and the GPU context stays usable. HEAT_ERR_ARG unless
+ * extra_arrivals is 0 or 1 and 0 <= limit_s <= 60. heat_debug_loop_wait(0, 0)
+ * restores the defaults. */
 heat_status heat_debug_loop_wait(unsigned int extra_arrivals, double limit_s);
 
 /* ---- operator-level entry points (device pointers, sim stream) ---------- */
@@ -607,9 +608,10 @@ heat_status heat_tuning_set(const heat_tuning* t);
  * tick graph of its engine, about `reps` iterations after 8 warm-up ones,
  * every iteration on a seeded residual that does not converge) for every
  * candidate (-1; the default form under the table's segment size; each other
- * variant with a segment size of 256, 512, 1024 or 2048 nodes; then, for the two fastest variants, the segment sizes whose work
- * items fill whole waves of resident blocks best; then the pointwise item
- * sizes and the persistent iteration) on this simulation's mesh and
+ * variant with a segment size of 256, 512, 1024 or 2048 nodes; then, for the
+ * two fastest variants, the segment sizes whose work items fill whole waves of
+ * resident blocks best; then the pointwise item sizes and the persistent
+ * iteration) on this simulation's mesh and
  * precision, and store the
  * fastest in the table entries of that precision and of the mesh's size
  * bucket. Outputs the resulting table and the winner's mean ms per iteration

@@ -161,8 +161,8 @@ static const WVariant kVariants[] = {
 constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
 
 // Process-wide tuning table, read when an engine is created: the warp apply
-// variant per precision (-1: FP32 the block-tile apply, FP64 the default form) and the segment tile size
-// per mesh-size bucket. Both are fixed per simulation size, so results stay
+// variant per precision (-1: FP32 the block-tile apply, FP64 the default form)
+// and the segment tile size per mesh-size bucket. Both are fixed per simulation size, so results stay
 // bitwise identical alone and in batches built under the same table.
 constexpr int kAutoSeg = 512;  // the default segment size: under the default variants, levels per tile from pick_levels
 static Tuning g_tuning = {{-1, 0, 0}, {kAutoSeg, kAutoSeg, kAutoSeg}, {2, 4, 4}, {2, 2, 2}, {0, 0, 0}};
@@ -966,7 +966,6 @@ heat_status engine_create(heat_sim* const* sims, int nsims, int precision, cudaS
     }
   e->ncheb = members_ncheb(e);
   e->tuning = tun ? *tun : tuning_get();
-  e->ks = kernel_set(precision, e->tuning, e->ncheb > 0, e->elem);
   e->stream = stream;
   // Capacities: the geometry is a function of each mesh and of whether the
   // member takes Chebyshev passes (they run on 16-lane segments where the plain
@@ -976,6 +975,7 @@ heat_status engine_create(heat_sim* const* sims, int nsims, int precision, cudaS
   size_t cap_res = 0;
   const KernelSet sets[2] = {kernel_set(precision, e->tuning, false, e->elem),
                              kernel_set(precision, e->tuning, true, e->elem)};
+  e->ks = sets[e->ncheb > 0 ? 1 : 0];
   const bool one_set = sets[0].apply_w == sets[1].apply_w && sets[0].dual == sets[1].dual && sets[0].res == sets[1].res;
   struct Need {
     int nx = 0, ny = 0, nz = 0;
